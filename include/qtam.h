@@ -97,8 +97,7 @@ typedef struct {
   int32_t n_q;            /* 1 .. 64 */
   double f_min, f_max;    /* log grid f_k = f_min (f_max/f_min)^(k/(K-1)), endpoints included */
   int32_t rows_per_plane; /* K >= 1 */
-  int32_t window;         /* QTAM_WIN_*; non-bisquare windows read a per-plan W' table (compile-time
-                             row variants with F32 envelopes, else the runtime engine) */
+  int32_t window;         /* QTAM_WIN_*; non-bisquare windows read a per-plan W' table */
   int32_t norm;           /* QTAM_NORM_* */
   double q_width;         /* half-width h = floor(f T q_width / Q); <= 0 selects sqrt(11) */
   double max_window_hz;   /* 0: automatic clamp from the largest centre gap (App. A); > 0: manual */
@@ -137,10 +136,9 @@ typedef struct {
    * division (qtam_inverse_single_tile).  remodulate = 1 multiplies the
    * envelopes by exp(+2 pi i k_c n / M): the undemodulated tile, i.e. the
    * inverse DFT of the unshifted filtered spectrum X W_k.  Both run on the
-   * CUDA cores: the compile-time row variants built for the dense mode
-   * where the length has them (FP32 compute, any envelope storage;
-   * M = 4320), else
-   * the runtime engine, which also serves the single-tile inverse;
+   * CUDA cores: the row variants registered for the dense mode where the
+   * length has them (FP32 compute, any envelope storage; M = 4320), else
+   * the length's own kernels, which also serve the single-tile inverse;
    * remodulate combined with short_dft = TENSOR, or eps with it, is
    * QTAM_ERR_UNSUPPORTED_SIZE. */
   double stopband_eps;
@@ -164,7 +162,7 @@ typedef struct {
   double kappa;                   /* max over kept bins of max_k W_k / P (all planes) */
   int64_t kept_bins;              /* |F_tau| for all planes */
   int64_t device_bytes;           /* bytes of resident plan tables on the device */
-  int32_t row_variant;            /* CUDA-core row-kernel variant in use (-1: runtime engine); with
+  int32_t row_variant;            /* CUDA-core row-kernel variant in use (-1: the length's own kernels); with
                                      the tensor-core short DFT it serves only an inverse of
                                      envelopes that are not 16-byte aligned */
   int32_t short_dft;              /* QTAM_SHORT_DFT_* engine of the envelope stage */

@@ -21,7 +21,9 @@ LIBNAME = "libqtam.so"
 SOURCES = ["qtam_api.cu", "kernels_long.cu", "kernels_rows.cu", "qtam_noalloc.cu", "qtam_stream.cu",
            "kernels_tc.cu", "kernels_rows_stream.cu", "kernels_rows_dense.cu", "kernels_rows_pair.cu",
            "kernels_rows_tuned.cu"]
-HEADERS = ["fft_core.cuh", "fft_static.cuh", "qtam_internal.h", "tc_sm100.cuh", "rows_common.cuh", "pair_fft.cuh"]
+PARTS = 8                      # kernels_any.cu compiles once per part (QTAM_PART), in parallel
+HEADERS = ["fft_core.cuh", "fft_static.cuh", "qtam_internal.h", "tc_sm100.cuh", "rows_common.cuh", "pair_fft.cuh",
+           "rows_any.cuh", "row_shapes.inc", "kernels_any.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
                 "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include")]
@@ -69,11 +71,13 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     cc = nvcc()
     objs = []
     jobs = []
-    with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
-        for s in SOURCES:
-            obj = os.path.join(BUILDDIR, s.replace(".cu", ".o"))
+    units = [("kernels_any.cu", f"kernels_any_{k}.o", [f"-DQTAM_PART={k}"]) for k in range(PARTS)]
+    units += [(s, s.replace(".cu", ".o"), []) for s in SOURCES]
+    with cf.ThreadPoolExecutor(max_workers=max(2, os.cpu_count() or 2)) as ex:
+        for src, name, defs in units:
+            obj = os.path.join(BUILDDIR, name)
             objs.append(obj)
-            cmd = [cc, *FLAGS, *extra_flags, "-c", os.path.join(CSRC, s), "-o", obj]
+            cmd = [cc, *FLAGS, *defs, *extra_flags, "-c", os.path.join(CSRC, src), "-o", obj]
             jobs.append(ex.submit(_run, cmd, verbose))
         outs = [j.result() for j in jobs]
     if verbose:

@@ -292,8 +292,14 @@ template <int S> struct Dft<20, S> : DftPFA<4, 5, S> {};
 template <int S> struct Dft<24, S> : DftPFA<8, 3, S> {};
 template <int S> struct Dft<25, S> : DftComposite<5, 5, S> {};
 template <int S> struct Dft<27, S> : DftComposite<3, 9, S> {};
+template <int S> struct Dft<30, S> : DftPFA<2, 15, S> {};
 template <int S> struct Dft<32, S> : DftComposite<4, 8, S> {};
+template <int S> struct Dft<36, S> : DftPFA<4, 9, S> {};
+template <int S> struct Dft<40, S> : DftPFA<8, 5, S> {};
+template <int S> struct Dft<45, S> : DftPFA<9, 5, S> {};
 template <int S> struct Dft<48, S> : DftPFA<16, 3, S> {};
+template <int S> struct Dft<50, S> : DftPFA<2, 25, S> {};
+template <int S> struct Dft<54, S> : DftPFA<2, 27, S> {};
 template <int S> struct Dft<64, S> : DftComposite<8, 8, S> {};
 template <int S> struct Dft<60, S> : DftPFA<4, 15, S> {};
 template <int S> struct Dft<75, S> : DftPFA<3, 25, S> {};

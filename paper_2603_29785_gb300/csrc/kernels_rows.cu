@@ -15,8 +15,10 @@
 // by sqrt(N/M), weights by c_k W'(d) and adds the result into the spectrum
 // accumulator A[k_c + d] with vector atomics (A stays L2-resident).
 //
-// The FFT itself is either the runtime engine (any 2^a 3^b 5^c length) or a
-// compile-time engine registered below for the lengths the workloads use.
+// FP32 plans run compile-time FFTs: a variant registered below for the lengths
+// the workloads use, or the length's own shape (kernels_any.cu: every length a
+// plan can have, with every window, storage type and dense-mode option).  FP64
+// plans run the runtime mixed-radix engine.
 #include "rows_common.cuh"
 
 namespace qtam {
@@ -188,13 +190,52 @@ const RowVariant* row_variant(int i) {
   return tuned_row_variant(i - pair_row_variant_count());
 }
 
+#define QTAM_PARTS(X) X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7)
+#define QTAM_DECL(k) const AnyShape* any_shapes_##k(int* count);
+QTAM_PARTS(QTAM_DECL)
+#undef QTAM_DECL
+const AnyShape* any_shape(int M) {
+  using Part = const AnyShape* (*)(int*);
+#define QTAM_NAME(k) any_shapes_##k,
+  static const Part parts[] = {QTAM_PARTS(QTAM_NAME)};
+#undef QTAM_NAME
+  for (Part part : parts) {
+    int n = 0;
+    const AnyShape* s = part(&n);
+    for (int i = 0; i < n; ++i)
+      if (s[i].M == M) return &s[i];
+  }
+  return nullptr;
+}
+#undef QTAM_PARTS
+
+namespace {
+// what forward and inverse launches of the length's own kernels share
+AnyArgs<float> any_args(const RowCfg& c, const RowDev<float>* rows, int n_rows, int n_sel, int64_t Nr, int env, int64_t B,
+                        const float2* twM, const float* wtab) {
+  AnyArgs<float> g{};
+  g.rows = rows;
+  g.sel = fast_div((uint32_t)n_sel);
+  g.n_rows = n_rows;
+  g.n_units = (uint32_t)(B * n_sel);
+  g.Nr = Nr;
+  g.tws = static_cast<const float2*>(c.any_tw);
+  g.wtab = wtab;
+  g.twM = twM;
+  g.env = env;
+  g.mode = c.floor ? (c.remod ? ANY_ABS : ANY_DENSE) : wtab ? ANY_TABLE : ANY_BISQUARE;
+  g.carrier = c.remod && g.mode != ANY_ABS;
+  return g;
+}
+// the kernels built for FP32 envelopes and bisquare bands serve the launch
+bool plain(const AnyArgs<float>& g) { return g.env == ENV_F32 && g.mode == ANY_BISQUARE && !g.carrier && !g.divide; }
+}  // namespace
+
 template <typename T>
 cudaError_t launch_rows_forward(const RowCfg& c, const RowDev<T>* rows, int n_rows, int64_t Nr, const cplx<T>* X,
                                 void* y, int env, int64_t B, const cplx<T>* twM, cudaStream_t st, const T* wtab) {
   const int64_t units = B * n_rows;
   if (units == 0) return cudaSuccess;
-  DenseArgs<T> da;
-  da.remod = c.remod;
   if constexpr (sizeof(T) == 4) {
     if (const RowVariant* v = row_variant(c.variant)) {
       const float2* stw = static_cast<const float2*>(c.stw);
@@ -206,32 +247,22 @@ cudaError_t launch_rows_forward(const RowCfg& c, const RowDev<T>* rows, int n_ro
         if (env == ENV_F32 && v->fwd_tab) return v->fwd_tab(rows, n_rows, Nr, X, y, B, stw, st, wtab);
       }
     }
-  }
-  GenericEngine eng{c.rp};
-  const unsigned blocks = (unsigned)units;
-  if constexpr (sizeof(T) == 4) {
-    switch (env) {
-      case ENV_BF16:
-        allow_smem((const void*)k_rows_forward<T, ENV_BF16>, c.smem);
-        k_rows_forward<T, ENV_BF16><<<blocks, c.threads, c.smem, st>>>(eng, rows, n_rows, Nr, X,
-                                                                       static_cast<__nv_bfloat162*>(y), units, twM, wtab, da);
-        break;
-      case ENV_F16:
-        allow_smem((const void*)k_rows_forward<T, ENV_F16>, c.smem);
-        k_rows_forward<T, ENV_F16><<<blocks, c.threads, c.smem, st>>>(eng, rows, n_rows, Nr, X,
-                                                                      static_cast<__half2*>(y), units, twM, wtab, da);
-        break;
-      default:
-        allow_smem((const void*)k_rows_forward<T, ENV_F32>, c.smem);
-        k_rows_forward<T, ENV_F32><<<blocks, c.threads, c.smem, st>>>(eng, rows, n_rows, Nr, X,
-                                                                      static_cast<float2*>(y), units, twM, wtab, da);
-    }
+    AnyArgs<float> g = any_args(c, rows, n_rows, n_rows, Nr, env, B, twM, wtab);
+    g.X = X;
+    g.y = y;
+    if (!plain(g)) return c.any->fwd_any(g, st);
+    g.tws = static_cast<const float2*>(c.any_tw_plain);
+    return c.any->fwd_plain(g, st);
   } else {
-    allow_smem((const void*)k_rows_forward<T, ENV_F64>, c.smem);
-    k_rows_forward<T, ENV_F64><<<blocks, c.threads, c.smem, st>>>(eng, rows, n_rows, Nr, X,
-                                                                  static_cast<double2*>(y), units, twM, wtab, da);
+    GenericEngine eng{c.rp};
+    DenseArgs<T> da;
+    da.remod = c.remod;
+    const cudaError_t e = allow_smem((const void*)k_rows_forward<T, ENV_F64>, c.smem);
+    if (e != cudaSuccess) return e;
+    k_rows_forward<T, ENV_F64><<<(unsigned)units, c.threads, c.smem, st>>>(eng, rows, n_rows, Nr, X,
+                                                                           static_cast<double2*>(y), units, twM, wtab, da);
+    return cudaGetLastError();
   }
-  return cudaGetLastError();
 }
 
 template <typename T>
@@ -253,32 +284,21 @@ cudaError_t launch_rows_inverse(const RowCfg& c, const RowDev<T>* rows, const in
         if (env == ENV_F32 && v->inv_tab) return v->inv_tab(rows, row_list, n_sel, n_rows, Nr, y, A, B, stw, st, wtab);
       }
     }
-  }
-  GenericEngine eng{c.rp};
-  const unsigned blocks = (unsigned)units;
-  if constexpr (sizeof(T) == 4) {
-    switch (env) {
-      case ENV_BF16:
-        allow_smem((const void*)k_rows_inverse<T, ENV_BF16>, c.smem);
-        k_rows_inverse<T, ENV_BF16><<<blocks, c.threads, c.smem, st>>>(
-            eng, rows, row_list, n_sel, n_rows, Nr, static_cast<const __nv_bfloat162*>(y), A, units, twM, wtab, da);
-        break;
-      case ENV_F16:
-        allow_smem((const void*)k_rows_inverse<T, ENV_F16>, c.smem);
-        k_rows_inverse<T, ENV_F16><<<blocks, c.threads, c.smem, st>>>(
-            eng, rows, row_list, n_sel, n_rows, Nr, static_cast<const __half2*>(y), A, units, twM, wtab, da);
-        break;
-      default:
-        allow_smem((const void*)k_rows_inverse<T, ENV_F32>, c.smem);
-        k_rows_inverse<T, ENV_F32><<<blocks, c.threads, c.smem, st>>>(
-            eng, rows, row_list, n_sel, n_rows, Nr, static_cast<const float2*>(y), A, units, twM, wtab, da);
-    }
+    AnyArgs<float> g = any_args(c, rows, n_rows, n_sel, Nr, env, B, twM, wtab);
+    g.row_list = row_list;
+    g.A = A;
+    g.y = const_cast<void*>(y);
+    g.divide = da.divide;
+    g.scale = da.scale;
+    return plain(g) ? c.any->inv_plain(g, st) : c.any->inv_any(g, st);
   } else {
-    allow_smem((const void*)k_rows_inverse<T, ENV_F64>, c.smem);
-    k_rows_inverse<T, ENV_F64><<<blocks, c.threads, c.smem, st>>>(
+    GenericEngine eng{c.rp};
+    const cudaError_t e = allow_smem((const void*)k_rows_inverse<T, ENV_F64>, c.smem);
+    if (e != cudaSuccess) return e;
+    k_rows_inverse<T, ENV_F64><<<(unsigned)units, c.threads, c.smem, st>>>(
         eng, rows, row_list, n_sel, n_rows, Nr, static_cast<const double2*>(y), A, units, twM, wtab, da);
+    return cudaGetLastError();
   }
-  return cudaGetLastError();
 }
 
 template cudaError_t launch_rows_forward<float>(const RowCfg&, const RowDev<float>*, int, int64_t, const float2*, void*,

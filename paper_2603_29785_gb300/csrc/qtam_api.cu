@@ -201,6 +201,8 @@ struct qtam_plan_s {
   void* d_tcA = nullptr;    // tensor-core short DFT operands (short_dft = TENSOR)
   void* d_tcAi = nullptr;
   void* d_tcG = nullptr;
+  void* d_any_tw = nullptr; // stage twiddles of the length's own shapes
+  void* d_any_tw_plain = nullptr;
   void* d_ones = nullptr;   // dense mode: 1/P := 1 for the single-tile inverse
   size_t device_bytes = 0;
   std::map<int, void*> variant_tw;   // stage twiddle tables per row-kernel variant
@@ -479,7 +481,7 @@ template <typename T> qtam_status upload_tables(qtam_plan_s* pl) {
   }
   if (!pl->all_bisquare()) {
     // one W'(0..h) table per distinct (window, parameter, half-width), read by
-    // the runtime engine; bisquare rows of a mixed bank keep the formula
+    // the row kernels; bisquare rows of a mixed bank keep the formula
     std::map<std::tuple<int, double, int>, int> off;
     std::vector<T> tab;
     for (size_t r = 0; r < rows.size(); ++r) {
@@ -499,6 +501,11 @@ template <typename T> qtam_status upload_tables(qtam_plan_s* pl) {
   if ((s = upload(&pl->d_rows, rows.data(), rows.size() * sizeof(RowDev<T>), tot)) != QTAM_OK) return s;
   if (pl->rc.tensor && (s = upload_tc_tables(pl, tot)) != QTAM_OK) return s;
   if (sizeof(T) == 4) {
+    const AnyShape* sh = pl->rc.any;
+    if ((s = upload_stage_table(sh->r, sh->nst, &pl->d_any_tw, tot)) != QTAM_OK) return s;
+    if ((s = upload_stage_table(sh->r_plain, sh->nst_plain, &pl->d_any_tw_plain, tot)) != QTAM_OK) return s;
+    pl->rc.any_tw = pl->d_any_tw;
+    pl->rc.any_tw_plain = pl->d_any_tw_plain;
     for (int v = 0; v < row_variant_count(); ++v) {
       const RowVariant* rv = row_variant(v);
       if (rv->M != pl->M) continue;
@@ -548,6 +555,8 @@ void free_plan(qtam_plan_s* pl) {
     cudaFree(pl->d_tcAi);
     cudaFree(pl->d_tcG);
     cudaFree(pl->d_ones);
+    cudaFree(pl->d_any_tw);
+    cudaFree(pl->d_any_tw_plain);
     cudaFree(pl->d_stw_col);
     cudaFree(pl->d_stw_row);
     for (auto& kv : pl->variant_tw) cudaFree(kv.second);
@@ -885,6 +894,7 @@ qtam_status qtam_plan(const qtam_plan_desc* d, int device, qtam_plan_t* out) {
   }
   pl->rc.tensor = pl->short_dft == QTAM_SHORT_DFT_TENSOR && tc_forward_supported(pl->M);
   pl->rc.remod = pl->remod;
+  pl->rc.floor = pl->eps > 0;
   pl->rc.dense = (pl->eps > 0 && pl->remod) ? 2 : (pl->eps > 0 || pl->remod) ? 1 : 0;
   if (!dbl) {
     // the first usable variant marked preferred for this length, else the
@@ -896,7 +906,8 @@ qtam_status qtam_plan(const qtam_plan_desc* d, int device, qtam_plan_t* out) {
           break;
         }
   }
-  if (pl->rc.threads > kMaxThreads || pl->rc.smem > (size_t)kMaxSmem) {
+  pl->rc.any = any_shape(pl->M);
+  if (pl->rc.threads > kMaxThreads || pl->rc.smem > (size_t)kMaxSmem || !pl->rc.any) {
     free_plan(pl);
     return fail(QTAM_ERR_UNSUPPORTED_SIZE, "n_out too large for one thread block");
   }
@@ -1000,7 +1011,7 @@ qtam_status qtam_plan_set_variant(qtam_plan_t pl, int32_t id) {
 
 qtam_status qtam_variant_describe(int32_t id, char* name, size_t capacity, int32_t* threads, int32_t* rows_per_block) {
   if (id == -1) {
-    if (name && capacity) std::snprintf(name, capacity, "runtime mixed-radix engine");
+    if (name && capacity) std::snprintf(name, capacity, "the length's own kernels");
     if (threads) *threads = 0;
     if (rows_per_block) *rows_per_block = 1;
     return QTAM_OK;

@@ -61,12 +61,69 @@ struct LongCfg {
   size_t col_smem, row_smem;
 };
 
+enum EnvKind { ENV_F32 = 0, ENV_F64 = 1, ENV_BF16 = 2, ENV_F16 = 3 };
+
+// Division of n < 2^31 by a launch constant d: floor(n m / 2^(31 + l)), l = ceil(log2 d),
+// m = floor(2^(31 + l) / d) + 1, exact because m d - 2^(31 + l) <= d <= 2^l.
+struct FastDiv {
+  uint32_t d, m, s;
+};
+inline FastDiv fast_div(uint32_t d) {
+  uint32_t l = 0;
+  while (l < 31 && (1u << l) < d) ++l;
+  return FastDiv{d, (uint32_t)(((uint64_t)1 << (31 + l)) / d + 1), l ? l - 1 : 0};
+}
+// Which weights and placement the rows of a launch use.
+enum AnyMode {
+  ANY_BISQUARE = 0,   // every row a bisquare band at baseband
+  ANY_TABLE = 1,      // bands at baseband, some rows with a window table
+  ANY_DENSE = 2,      // stopband floor: every bin of the spectrum, at baseband
+  ANY_ABS = 3,        // floor and carrier: bins at their own positions
+};
+
+template <typename T> struct AnyArgs {
+  const RowDev<T>* rows;
+  const int* row_list;      // inverse: selected rows
+  FastDiv sel;              // rows per segment (forward: all, inverse: selected)
+  int n_rows;
+  uint32_t n_units;
+  int64_t Nr;
+  const cplx<T>* X;         // forward: spectra
+  cplx<T>* A;               // inverse: accumulators
+  void* y;                  // envelopes (inverse: read only)
+  const cplx<T>* tws;       // stage twiddles of the shape
+  const T* wtab;
+  const cplx<T>* twM;       // M-point table (carrier)
+  int env;                  // EnvKind of y
+  int mode;                 // AnyMode
+  int carrier;              // envelopes times e^{+2 pi i k_c n / M}
+  int divide;               // inverse: X = S scale / w instead of A += w S
+  T scale;
+};
+
+// Kernels of one envelope length (kernels_any.cu, FP32 arithmetic): `*_plain`
+// for FP32 envelopes and bisquare bands, `*_any` for every storage type, window
+// and dense-mode option.  The plain forward rows have their own radix sequence.
+using AnyFn = cudaError_t (*)(const AnyArgs<float>&, cudaStream_t);
+struct AnyShape {
+  int M;
+  int nst_plain, nst;
+  int r_plain[kMaxStages], r[kMaxStages];
+  AnyFn fwd_plain, inv_plain, fwd_any, inv_any;
+};
+// the shape of length M, or nullptr: every 2^a 3^b 5^c from 3 to 7680, and 8192
+const AnyShape* any_shape(int M);
+
 struct RowCfg {
-  RadixPlan rp;  // radices of M (runtime engine)
+  RadixPlan rp;  // radices of M (runtime engine, FP64)
   int threads;
   size_t smem;
-  int variant;   // index of a compile-time row-kernel variant, -1 = runtime engine
+  int variant;   // index of a registered row-kernel variant, -1 = the length's own shape
+  const AnyShape* any = nullptr;   // that shape (FP32 plans) ...
+  const void* any_tw = nullptr;    // ... and its stage twiddles,
+  const void* any_tw_plain = nullptr;   // those of the plain forward rows
   int remod = 0; // dense mode: remodulated envelopes
+  int floor = 0; // dense mode: stopband floor
   int dense = 0; // stopband floor or carrier: only the variants' dense kernels serve the plan;
                  // 2: floor and carrier (tiles span the spectrum, bins at their own positions)
   const void* stw = nullptr;   // stage twiddle tables of that variant
@@ -79,7 +136,6 @@ struct RowCfg {
   const void* tcG = nullptr;
 };
 
-enum EnvKind { ENV_F32 = 0, ENV_F64 = 1, ENV_BF16 = 2, ENV_F16 = 3 };
 
 // Tensor-core rows (kernels_tc.cu): M must be 8192, FP32 compute.
 bool tc_forward_supported(int M);

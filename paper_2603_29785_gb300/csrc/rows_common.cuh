@@ -69,15 +69,15 @@ template <> struct Env<double2, ENV_F64> {
 // i >= M + dlo.  The weight is c W'(d) = (kw (h^2 - d^2))^2 with
 // kw = sqrt(c)/h^2; with FEXACT (h < 4096) h^2 - d^2 is formed exactly in
 // floating point, otherwise as the integer product (h - |d|)(h + |d|).  The
-// other App. A windows (runtime engine only) read W'(|d|) from a per-plan
+// other App. A windows read W'(|d|) from a per-plan
 // table instead; positions outside the band read W'(h) and are multiplied
 // by a zero bin.
 template <typename T, bool FEXACT> struct RowCtx {
   int kc, h, M, dhi, mlo;
   T kw, h2;
-  const T* wt;   // runtime engine only: W'(0..h) table of a non-bisquare window, or null
+  const T* wt;   // W'(0..h) table of a non-bisquare window, or null
   T cw;          // its normalisation (c_fwd or c_inv)
-  T ew;          // runtime engine only: weight where the window vanishes (dense mode), else 0
+  T ew;          // weight where the window vanishes (dense mode), else 0
   __device__ __forceinline__ void locate(int i, bool& in, int& d) const {
     const bool lo = i <= dhi;
     in = lo || i >= mlo;
