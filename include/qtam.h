@@ -162,9 +162,9 @@ typedef struct {
   double kappa;                   /* max over kept bins of max_k W_k / P (all planes) */
   int64_t kept_bins;              /* |F_tau| for all planes */
   int64_t device_bytes;           /* bytes of resident plan tables on the device */
-  int32_t row_variant;            /* CUDA-core row-kernel variant in use (-1: the length's own kernels); with
-                                     the tensor-core short DFT it serves only an inverse of
-                                     envelopes that are not 16-byte aligned */
+  int32_t row_variant;            /* registered CUDA-core row variant of the plan's length (its first choice
+                                     before tuning), -1 if none; launches run the length's own
+                                     kernels until qtam_plan_set_variant chooses a variant */
   int32_t short_dft;              /* QTAM_SHORT_DFT_* engine of the envelope stage */
   double stopband_eps;            /* dense mode floor (0: off) */
   int32_t remodulate;             /* 1: envelopes carry the carrier exp(+2 pi i k_c n / M) */
@@ -191,9 +191,10 @@ QTAM_API qtam_status qtam_plan_rows(qtam_plan_t plan, double* f, int64_t* kc, in
  * plane p; 0 = all planes), FP64, into the caller's host array of N/2+1. */
 QTAM_API qtam_status qtam_frame_operator(qtam_plan_t plan, uint64_t plane_mask, double* p_out);
 
-/* Row-kernel variants (launch shapes) usable for this plan: the runtime
- * mixed-radix engine (-1, any length) and the compile-time variants built for
- * the plan's envelope length M (FP32 compute).  Writes up to `capacity` ids
+/* Row-kernel variants (launch shapes) usable for this plan: the kernels of the
+ * plan's own length (-1, the ones a new plan runs; the runtime mixed-radix
+ * engine for FP64 compute) and the variants registered for that length (FP32
+ * compute).  Writes up to `capacity` ids
  * into `ids` and the total into *count.  All variants compute the same
  * transform; they differ in radix sequence, rows per block and occupancy.
  * An autotuner times them (qtam_stage_envelopes / qtam_stage_accumulate)

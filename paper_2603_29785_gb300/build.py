@@ -19,7 +19,7 @@ LIBDIR = os.path.join(HERE, "lib")
 BUILDDIR = os.path.join(LIBDIR, "_build")
 LIBNAME = "libqtam.so"
 SOURCES = ["qtam_api.cu", "kernels_long.cu", "kernels_rows.cu", "qtam_noalloc.cu", "qtam_stream.cu",
-           "kernels_tc.cu", "kernels_rows_stream.cu", "kernels_rows_dense.cu", "kernels_rows_pair.cu",
+           "kernels_tc.cu", "kernels_rows_dense.cu", "kernels_rows_pair.cu",
            "kernels_rows_tuned.cu"]
 PARTS = 8                      # kernels_any.cu compiles once per part (QTAM_PART), in parallel
 HEADERS = ["fft_core.cuh", "fft_static.cuh", "qtam_internal.h", "tc_sm100.cuh", "rows_common.cuh", "pair_fft.cuh",

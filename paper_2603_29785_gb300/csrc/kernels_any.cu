@@ -19,8 +19,16 @@ template <class Plain, class Sh> AnyShape make_shape() {
   s.nst = Sh::sequence(s.r);
   s.fwd_plain = launch_any_fwd<Plain, float, ENV_F32, ANY_BISQUARE>;
   s.inv_plain = launch_any_inv<Sh, float, ENV_F32, ANY_BISQUARE>;
-  s.fwd_any = launch_any_fwd<Sh, float, -1, -1>;
-  s.inv_any = launch_any_inv<Sh, float, -1, -1>;
+  s.fwd_stream = launch_any_fwd<Sh, float, ENV_F32, ANY_BISQUARE, true>;
+  s.inv_stream = launch_any_inv<Sh, float, ENV_F32, ANY_BISQUARE, true>;
+  s.fwd[0] = launch_any_fwd<Sh, float, -1, ANY_BISQUARE>;
+  s.inv[0] = launch_any_inv<Sh, float, -1, ANY_BISQUARE>;
+  s.fwd[1] = launch_any_fwd<Sh, float, -1, ANY_TABLE>;
+  s.inv[1] = launch_any_inv<Sh, float, -1, ANY_TABLE>;
+  s.fwd[2] = launch_any_fwd<Sh, float, -1, ANY_DENSE>;
+  s.inv[2] = launch_any_inv<Sh, float, -1, ANY_DENSE>;
+  s.fwd[3] = launch_any_fwd<Sh, float, -1, ANY_ABS>;
+  s.inv[3] = launch_any_inv<Sh, float, -1, ANY_ABS>;
   return s;
 }
 #define QTAM_SHAPE(...) make_shape<__VA_ARGS__>(),

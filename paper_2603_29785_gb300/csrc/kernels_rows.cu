@@ -15,10 +15,16 @@
 // by sqrt(N/M), weights by c_k W'(d) and adds the result into the spectrum
 // accumulator A[k_c + d] with vector atomics (A stays L2-resident).
 //
-// FP32 plans run compile-time FFTs: a variant registered below for the lengths
-// the workloads use, or the length's own shape (kernels_any.cu: every length a
-// plan can have, with every window, storage type and dense-mode option).  FP64
-// plans run the runtime mixed-radix engine.
+// FP32 plans run compile-time FFTs: the length's own shape (kernels_any.cu:
+// every length a plan can have, with every window, storage type and dense-mode
+// option), or a variant registered below once qtam_plan_set_variant chose it.
+// The own shapes are the default because they were faster than the best
+// registered variant, forward + inverse on a GB300: M = 4800 (64 segments x 640
+// rows) 450 + 490 against 488 + 483 us; 2400 (55 x 384) 111 + 123 against 115 +
+// 141; 1200 (48 x 384) 55 + 58 against 57 + 65; 600 (96 x 384) 47 + 55 against 51
+// + 60; 300 (128 x 384) 35 + 41 against 35 + 47; 150 (200 x 384) 29 + 35 against
+// 33 + 45; 75 (400 x 384) 45 + 37 against 49 + 62; 8192 (16 x 640) 248 + 201
+// against 252 + 230.  FP64 plans run the runtime mixed-radix engine.
 #include "rows_common.cuh"
 
 namespace qtam {
@@ -237,7 +243,7 @@ cudaError_t launch_rows_forward(const RowCfg& c, const RowDev<T>* rows, int n_ro
   const int64_t units = B * n_rows;
   if (units == 0) return cudaSuccess;
   if constexpr (sizeof(T) == 4) {
-    if (const RowVariant* v = row_variant(c.variant)) {
+    if (const RowVariant* v = c.chosen ? row_variant(c.variant) : nullptr) {
       const float2* stw = static_cast<const float2*>(c.stw);
       if (c.dense) {
         if (v->fwd_dense)
@@ -250,7 +256,7 @@ cudaError_t launch_rows_forward(const RowCfg& c, const RowDev<T>* rows, int n_ro
     AnyArgs<float> g = any_args(c, rows, n_rows, n_rows, Nr, env, B, twM, wtab);
     g.X = X;
     g.y = y;
-    if (!plain(g)) return c.any->fwd_any(g, st);
+    if (!plain(g)) return c.any->fwd[g.mode](g, st);
     g.tws = static_cast<const float2*>(c.any_tw_plain);
     return c.any->fwd_plain(g, st);
   } else {
@@ -273,7 +279,7 @@ cudaError_t launch_rows_inverse(const RowCfg& c, const RowDev<T>* rows, const in
   da.remod = c.remod;
   if (units == 0) return cudaSuccess;
   if constexpr (sizeof(T) == 4) {
-    if (const RowVariant* v = da.divide ? nullptr : row_variant(c.variant)) {
+    if (const RowVariant* v = c.chosen && !da.divide ? row_variant(c.variant) : nullptr) {
       const float2* stw = static_cast<const float2*>(c.stw);
       if (c.dense) {
         if (v->inv_dense)
@@ -290,7 +296,7 @@ cudaError_t launch_rows_inverse(const RowCfg& c, const RowDev<T>* rows, const in
     g.y = const_cast<void*>(y);
     g.divide = da.divide;
     g.scale = da.scale;
-    return plain(g) ? c.any->inv_plain(g, st) : c.any->inv_any(g, st);
+    return plain(g) ? c.any->inv_plain(g, st) : c.any->inv[g.mode](g, st);
   } else {
     GenericEngine eng{c.rp};
     const cudaError_t e = allow_smem((const void*)k_rows_inverse<T, ENV_F64>, c.smem);
@@ -299,6 +305,36 @@ cudaError_t launch_rows_inverse(const RowCfg& c, const RowDev<T>* rows, const in
         eng, rows, row_list, n_sel, n_rows, Nr, static_cast<const double2*>(y), A, units, twM, wtab, da);
     return cudaGetLastError();
   }
+}
+
+cudaError_t launch_rows_stream_forward(const RowCfg& c, const RowDev<float>* rows, int n_rows, int64_t Nr, const float2* X,
+                                       float2* y, int64_t pitch, int Gm, int Hn, const float2* phase, int64_t B,
+                                       cudaStream_t st) {
+  if (B * n_rows == 0) return cudaSuccess;
+  AnyArgs<float> g = any_args(c, rows, n_rows, n_rows, Nr, ENV_F32, B, nullptr, nullptr);
+  g.X = X;
+  g.y = y;
+  g.pitch = pitch;
+  g.Gm = Gm;
+  g.Hn = Hn;
+  g.phase = phase;
+  return c.any->fwd_stream(g, st);
+}
+cudaError_t launch_rows_stream_inverse(const RowCfg& c, const RowDev<float>* rows, const int* row_list, int n_sel,
+                                       int n_rows, int64_t Nr, const float2* hist, int hcols, const float2* ynew,
+                                       int64_t pitch, int Hn, const float2* phase, float2* A, int64_t B,
+                                       cudaStream_t st) {
+  if (B * n_sel == 0) return cudaSuccess;
+  AnyArgs<float> g = any_args(c, rows, n_rows, n_sel, Nr, ENV_F32, B, nullptr, nullptr);
+  g.row_list = row_list;
+  g.A = A;
+  g.y = const_cast<float2*>(ynew);
+  g.hist = hist;
+  g.hcols = hcols;
+  g.pitch = pitch;
+  g.Hn = Hn;
+  g.phase = phase;
+  return c.any->inv_stream(g, st);
 }
 
 template cudaError_t launch_rows_forward<float>(const RowCfg&, const RowDev<float>*, int, int64_t, const float2*, void*,

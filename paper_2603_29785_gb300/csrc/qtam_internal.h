@@ -76,7 +76,7 @@ inline FastDiv fast_div(uint32_t d) {
 // Which weights and placement the rows of a launch use.
 enum AnyMode {
   ANY_BISQUARE = 0,   // every row a bisquare band at baseband
-  ANY_TABLE = 1,      // bands at baseband, some rows with a window table
+  ANY_TABLE = 1,      // bands at baseband, every row with a window table
   ANY_DENSE = 2,      // stopband floor: every bin of the spectrum, at baseband
   ANY_ABS = 3,        // floor and carrier: bins at their own positions
 };
@@ -97,19 +97,27 @@ template <typename T> struct AnyArgs {
   int env;                  // EnvKind of y
   int mode;                 // AnyMode
   int carrier;              // envelopes times e^{+2 pi i k_c n / M}
-  int divide;               // inverse: X = S scale / w instead of A += w S
+  int divide;               // dense inverse: X = S scale / w instead of A += w S
   T scale;
+  // streaming launches: y is the map (forward) or its new columns (inverse) of
+  // `pitch` columns a row; a chunk keeps the Hn columns from Gm on (Hn also its
+  // advance), times phase[chunk][row]; hist: the hcols columns before y
+  int64_t pitch;
+  int Gm, Hn;
+  const cplx<T>* phase;
+  const cplx<T>* hist;
+  int64_t hcols;
 };
 
-// Kernels of one envelope length (kernels_any.cu, FP32 arithmetic): `*_plain`
-// for FP32 envelopes and bisquare bands, `*_any` for every storage type, window
-// and dense-mode option.  The plain forward rows have their own radix sequence.
+// Kernels of one envelope length (kernels_any.cu, FP32 arithmetic): `plain` for
+// FP32 envelopes and bisquare bands, `stream` for the same with overlap-save
+// columns, fwd / inv [AnyMode] for every storage type.  The plain forward rows have their own radix sequence.
 using AnyFn = cudaError_t (*)(const AnyArgs<float>&, cudaStream_t);
 struct AnyShape {
   int M;
   int nst_plain, nst;
   int r_plain[kMaxStages], r[kMaxStages];
-  AnyFn fwd_plain, inv_plain, fwd_any, inv_any;
+  AnyFn fwd_plain, inv_plain, fwd_stream, inv_stream, fwd[4], inv[4];
 };
 // the shape of length M, or nullptr: every 2^a 3^b 5^c from 3 to 7680, and 8192
 const AnyShape* any_shape(int M);
@@ -118,7 +126,8 @@ struct RowCfg {
   RadixPlan rp;  // radices of M (runtime engine, FP64)
   int threads;
   size_t smem;
-  int variant;   // index of a registered row-kernel variant, -1 = the length's own shape
+  int variant;   // index of a registered row-kernel variant, -1 = none
+  int chosen = 0;   // launches run that variant (qtam_plan_set_variant), else the length's own shape
   const AnyShape* any = nullptr;   // that shape (FP32 plans) ...
   const void* any_tw = nullptr;    // ... and its stage twiddles,
   const void* any_tw_plain = nullptr;   // those of the plain forward rows
@@ -194,26 +203,10 @@ const RowVariant* pair_row_variant(int i);
 // the short lengths, a four-stage sequence at M = 8192
 int tuned_row_variant_count();
 const RowVariant* tuned_row_variant(int i);
-// Fused streaming row kernels (kernels_rows_stream.cu) of a compile-time
-// variant, looked up by the variant's name: forward with the crop-and-phase
-// store into the map, inverse with the history/new-columns chunk load.
-using StreamFwdFn = cudaError_t (*)(const RowDev<float>* rows, int n_rows, int64_t Nr, const float2* X, float2* y,
-                                    int64_t pitch, int Gm, int Hn, const float2* phase, int64_t B, const float2* twM,
-                                    cudaStream_t st);
-using StreamInvFn = cudaError_t (*)(const RowDev<float>* rows, const int* row_list, int n_sel, int n_rows, int64_t Nr,
-                                    const float2* hist, int hcols, const float2* ynew, int64_t pitch, int Hn,
-                                    const float2* phase, float2* A, int64_t B, const float2* twM, cudaStream_t st);
-struct StreamRowFns {
-  const char* name;
-  StreamFwdFn fwd;
-  StreamInvFn inv;
-};
-const StreamRowFns* stream_row_fns(const char* variant_name);
-
 // Streaming steps with the fused row kernels (qtam_api.cu, used by
 // qtam_stream.cu).  *used is false (and nothing is launched) when the plan
-// has no fused kernels: F32 compute and envelopes, bisquare windows, a
-// compile-time variant with a fused entry.  phase is [b][P K] complex FP32.
+// has no fused kernels (they serve F32 compute and envelopes and bisquare
+// windows).  phase is [b][P K] complex FP32.
 qtam_status stream_forward_fused(qtam_plan_s* pl, const void* x, int64_t b, void* ymap, int64_t pitch, int Gm, int Hn,
                                  const void* phase, void* ws, size_t wsb, cudaStream_t st, bool* used);
 qtam_status stream_inverse_fused(qtam_plan_s* pl, const void* hist, int hcols, const void* ynew, int64_t pitch, int Hn,
@@ -250,6 +243,16 @@ template <typename T>
 cudaError_t launch_rows_inverse(const RowCfg& c, const RowDev<T>* rows, const int* row_list, int n_sel, int n_rows,
                                 int64_t Nr, const void* y, int env, cplx<T>* A, int64_t B, const cplx<T>* twM,
                                 cudaStream_t st, const T* wtab = nullptr, DenseArgs<T> da = DenseArgs<T>());
+
+// The plain rows of a plan as overlap-save chunks: forward with a store that
+// writes only a chunk's kept columns, times its phase, into the map; inverse
+// with a load that assembles a chunk from the map history and the new columns.
+cudaError_t launch_rows_stream_forward(const RowCfg& c, const RowDev<float>* rows, int n_rows, int64_t Nr, const float2* X,
+                                       float2* y, int64_t pitch, int Gm, int Hn, const float2* phase, int64_t B,
+                                       cudaStream_t st);
+cudaError_t launch_rows_stream_inverse(const RowCfg& c, const RowDev<float>* rows, const int* row_list, int n_sel,
+                                       int n_rows, int64_t Nr, const float2* hist, int hcols, const float2* ynew,
+                                       int64_t pitch, int Hn, const float2* phase, float2* A, int64_t B, cudaStream_t st);
 
 // radix sequence of the static long-FFT engine used for a pass of length m
 // with 2^nbs interleaved transforms (FP32); false when the runtime engine runs

@@ -1,6 +1,5 @@
-// Shared templates of the per-row kernels (included by kernels_rows.cu and
-// kernels_rows_stream.cu, each translation unit instantiating its own
-// kernels): envelope storage conversions, the per-row context (band limits
+// Shared templates of the per-row kernels (each translation unit instantiates
+// its own kernels): envelope storage conversions, the per-row context (band limits
 // and window weight), band loads and envelope stores, the band accumulation,
 // the FFT engines (runtime mixed-radix and compile-time), and the forward /
 // inverse row bodies.

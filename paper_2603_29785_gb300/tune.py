@@ -31,7 +31,8 @@ def _key(plan: "qtam.Plan", batch: int) -> str:
     i, d = plan.info, plan._desc
     # the plan's kind: window (band_bins tells composite banks apart), dense-mode options, short-DFT engine
     kind = f"w{d.window}:{d.window_param}:{i['band_bins']}|eps{d.stopband_eps}|rm{d.remodulate}|sd{d.short_dft}"
-    return f"{name}|N{plan.N}|P{plan.P}|K{plan.K}|M{plan.M}|B{batch}|{plan.compute}/{plan.envelope}|{kind}"
+    # k2: choices timed before the lengths had kernels of their own (variant -1) do not count
+    return f"k2|{name}|N{plan.N}|P{plan.P}|K{plan.K}|M{plan.M}|B{batch}|{plan.compute}/{plan.envelope}|{kind}"
 
 
 def _load(path):
