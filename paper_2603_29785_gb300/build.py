@@ -21,9 +21,10 @@ LIBNAME = "libqtam.so"
 SOURCES = ["qtam_api.cu", "kernels_long.cu", "kernels_rows.cu", "qtam_noalloc.cu", "qtam_stream.cu",
            "kernels_tc.cu", "kernels_rows_dense.cu", "kernels_rows_pair.cu",
            "kernels_rows_tuned.cu"]
-PARTS = 8                      # kernels_any.cu compiles once per part (QTAM_PART), in parallel
+PARTS = 16                     # kernels_any.cu compiles once per part (QTAM_PART), in parallel
+LONG_PARTS = 4                 # and kernels_long_any.cu (QTAM_LONG_PART)
 HEADERS = ["fft_core.cuh", "fft_static.cuh", "qtam_internal.h", "tc_sm100.cuh", "rows_common.cuh", "pair_fft.cuh",
-           "rows_any.cuh", "row_shapes.inc", "kernels_any.cu"]
+           "rows_any.cuh", "row_shapes.inc", "kernels_any.cu", "pass_fft.cuh", "long_shapes.inc", "kernels_long_any.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
                 "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include")]
@@ -72,6 +73,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     objs = []
     jobs = []
     units = [("kernels_any.cu", f"kernels_any_{k}.o", [f"-DQTAM_PART={k}"]) for k in range(PARTS)]
+    units += [("kernels_long_any.cu", f"kernels_long_any_{k}.o", [f"-DQTAM_LONG_PART={k}"]) for k in range(LONG_PARTS)]
     units += [(s, s.replace(".cu", ".o"), []) for s in SOURCES]
     with cf.ThreadPoolExecutor(max_workers=max(2, os.cpu_count() or 2)) as ex:
         for src, name, defs in units:

@@ -274,7 +274,38 @@ void with_engine(const RadixPlan& rp, int nbs, int static_nbs, size_t gen_smem, 
     return true;                                    \
   }
 
+// one pass of a batch through its compile-time shape
+template <typename T>
+cudaError_t launch_shape(LongFn f, const LongCfg& c, bool cols, const cplx<T>* in, cplx<T>* out, int64_t nb, cudaStream_t st) {
+  if constexpr (sizeof(T) == 4) {
+    const LongPass g{c.n, cols ? c.n2 : c.n1, in, out, static_cast<const float2*>(c.tw4),
+                     static_cast<const float2*>(cols ? c.stw_col : c.stw_row)};
+    return f(g, (unsigned)nb, st);
+  } else {
+    return cudaErrorNotSupported;
+  }
+}
+
 }  // namespace
+
+#define QTAM_PARTS(X) X(0) X(1) X(2) X(3)
+#define QTAM_DECL(k) const LongShapeFns* long_shapes_##k(int* count);
+QTAM_PARTS(QTAM_DECL)
+#undef QTAM_DECL
+const LongShapeFns* long_shape(int M) {
+  using Part = const LongShapeFns* (*)(int*);
+#define QTAM_NAME(k) long_shapes_##k,
+  static const Part parts[] = {QTAM_PARTS(QTAM_NAME)};
+#undef QTAM_NAME
+  for (Part part : parts) {
+    int n = 0;
+    const LongShapeFns* s = part(&n);
+    for (int i = 0; i < n; ++i)
+      if (s[i].M == M) return &s[i];
+  }
+  return nullptr;
+}
+#undef QTAM_PARTS
 
 bool long_static_radices(int m, int nbs, int* r, int* nst) {
   if (nbs == 4) {
@@ -293,16 +324,26 @@ cudaError_t launch_spectrum(const LongCfg& c, const cplx<T>* z, cplx<T>* U, cplx
   for (int64_t s0 = 0; s0 < B; s0 += kMaxGridY) {
     const int64_t nb = (B - s0) < kMaxGridY ? (B - s0) : kMaxGridY;
     const int64_t off = s0 * c.n;
-    with_engine<T>(c.rp1, c.col_nbs, 4, c.col_smem, c.stw_col, twn, [&](auto eng, size_t smem, const cplx<T>* ftw) {
-      using E = decltype(eng);
-      dim3 g(c.n2 >> c.col_nbs, (unsigned)nb);
-      launch_pass(k_col_forward<E, T>, eng, smem, g, st, c.n, c.n2, z + off, U + off, tw4, ftw);
-    });
-    with_engine<T>(c.rp2, c.row_nbs, 2, c.row_smem, c.stw_row, twn, [&](auto eng, size_t smem, const cplx<T>* ftw) {
-      using E = decltype(eng);
-      dim3 g(c.n1 >> c.row_nbs, (unsigned)nb);
-      launch_pass(k_row_forward<E, T>, eng, smem, g, st, c.n, c.n1, (const cplx<T>*)(U + off), Z + off, ftw);
-    });
+    if (c.cols) {
+      const cudaError_t e = launch_shape<T>(c.cols->col_fwd, c, true, z + off, U + off, nb, st);
+      if (e != cudaSuccess) return e;
+    } else {
+      with_engine<T>(c.rp1, c.col_nbs, 4, c.col_smem, c.stw_col, twn, [&](auto eng, size_t smem, const cplx<T>* ftw) {
+        using E = decltype(eng);
+        dim3 g(c.n2 >> c.col_nbs, (unsigned)nb);
+        launch_pass(k_col_forward<E, T>, eng, smem, g, st, c.n, c.n2, z + off, U + off, tw4, ftw);
+      });
+    }
+    if (c.rows) {
+      const cudaError_t e = launch_shape<T>(c.rows->row_fwd, c, false, (const cplx<T>*)(U + off), Z + off, nb, st);
+      if (e != cudaSuccess) return e;
+    } else {
+      with_engine<T>(c.rp2, c.row_nbs, 2, c.row_smem, c.stw_row, twn, [&](auto eng, size_t smem, const cplx<T>* ftw) {
+        using E = decltype(eng);
+        dim3 g(c.n1 >> c.row_nbs, (unsigned)nb);
+        launch_pass(k_row_forward<E, T>, eng, smem, g, st, c.n, c.n1, (const cplx<T>*)(U + off), Z + off, ftw);
+      });
+    }
     dim3 g3((unsigned)((c.n / 2 + 1 + 256 * kUntanglePairs - 1) / (256 * kUntanglePairs)), (unsigned)nb);
     k_untangle_forward<T><<<g3, 256, 0, st>>>(c.n, Z + off, X + s0 * (int64_t)(c.n + 1), twN);
   }
@@ -319,16 +360,26 @@ cudaError_t launch_synthesis(const LongCfg& c, const cplx<T>* A, const T* invP, 
     dim3 g0((unsigned)((c.n / 2 + 1 + 256 * kUntanglePairs - 1) / (256 * kUntanglePairs)), (unsigned)nb);
     k_untangle_inverse<T><<<g0, 256, 0, st>>>(c.n, A + s0 * (int64_t)(c.n + 1), invP, Zi + off, twN,
                                               (T)1 / (T)c.n);
-    with_engine<T>(c.rp2, c.row_nbs, 2, c.row_smem, c.stw_row, twn, [&](auto eng, size_t smem, const cplx<T>* ftw) {
-      using E = decltype(eng);
-      dim3 g(c.n1 >> c.row_nbs, (unsigned)nb);
-      launch_pass(k_row_inverse<E, T>, eng, smem, g, st, c.n, c.n1, (const cplx<T>*)(Zi + off), Vb + off, tw4, ftw);
-    });
-    with_engine<T>(c.rp1, c.col_nbs, 4, c.col_smem, c.stw_col, twn, [&](auto eng, size_t smem, const cplx<T>* ftw) {
-      using E = decltype(eng);
-      dim3 g(c.n2 >> c.col_nbs, (unsigned)nb);
-      launch_pass(k_col_inverse<E, T>, eng, smem, g, st, c.n, c.n2, (const cplx<T>*)(Vb + off), xout + off, ftw);
-    });
+    if (c.rows) {
+      const cudaError_t e = launch_shape<T>(c.rows->row_inv, c, false, (const cplx<T>*)(Zi + off), Vb + off, nb, st);
+      if (e != cudaSuccess) return e;
+    } else {
+      with_engine<T>(c.rp2, c.row_nbs, 2, c.row_smem, c.stw_row, twn, [&](auto eng, size_t smem, const cplx<T>* ftw) {
+        using E = decltype(eng);
+        dim3 g(c.n1 >> c.row_nbs, (unsigned)nb);
+        launch_pass(k_row_inverse<E, T>, eng, smem, g, st, c.n, c.n1, (const cplx<T>*)(Zi + off), Vb + off, tw4, ftw);
+      });
+    }
+    if (c.cols) {
+      const cudaError_t e = launch_shape<T>(c.cols->col_inv, c, true, (const cplx<T>*)(Vb + off), xout + off, nb, st);
+      if (e != cudaSuccess) return e;
+    } else {
+      with_engine<T>(c.rp1, c.col_nbs, 4, c.col_smem, c.stw_col, twn, [&](auto eng, size_t smem, const cplx<T>* ftw) {
+        using E = decltype(eng);
+        dim3 g(c.n2 >> c.col_nbs, (unsigned)nb);
+        launch_pass(k_col_inverse<E, T>, eng, smem, g, st, c.n, c.n2, (const cplx<T>*)(Vb + off), xout + off, ftw);
+      });
+    }
   }
   return cudaGetLastError();
 }

@@ -196,7 +196,7 @@ const RowVariant* row_variant(int i) {
   return tuned_row_variant(i - pair_row_variant_count());
 }
 
-#define QTAM_PARTS(X) X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7)
+#define QTAM_PARTS(X) X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12) X(13) X(14) X(15)
 #define QTAM_DECL(k) const AnyShape* any_shapes_##k(int* count);
 QTAM_PARTS(QTAM_DECL)
 #undef QTAM_DECL

@@ -512,15 +512,23 @@ template <typename T> qtam_status upload_tables(qtam_plan_s* pl) {
       if ((s = upload_stage_table(rv->r, rv->nst, &p, tot, rv->tw_pair != 0)) != QTAM_OK) return s;
       pl->variant_tw[v] = p;
     }
+    // the passes of the long FFT: powers of two have their own engines
     int r[kMaxStages], nst = 0;
+    const LongShapeFns* ls = long_shape(pl->lc.n1);
     if (long_static_radices(pl->lc.n1, pl->lc.col_nbs, r, &nst)) {
       if ((s = upload_stage_table(r, nst, &pl->d_stw_col, tot)) != QTAM_OK) return s;
-      pl->lc.stw_col = pl->d_stw_col;
+    } else if (ls && ls->col_fwd) {
+      if ((s = upload_stage_table(ls->r, ls->nst, &pl->d_stw_col, tot)) != QTAM_OK) return s;
+      pl->lc.cols = ls;
     }
+    pl->lc.stw_col = pl->d_stw_col;
     if (long_static_radices(pl->lc.n2, pl->lc.row_nbs, r, &nst)) {
       if ((s = upload_stage_table(r, nst, &pl->d_stw_row, tot)) != QTAM_OK) return s;
-      pl->lc.stw_row = pl->d_stw_row;
+    } else if ((ls = long_shape(pl->lc.n2))) {
+      if ((s = upload_stage_table(ls->r, ls->nst, &pl->d_stw_row, tot)) != QTAM_OK) return s;
+      pl->lc.rows = ls;
     }
+    pl->lc.stw_row = pl->d_stw_row;
     auto it = pl->variant_tw.find(pl->rc.variant);
     pl->rc.stw = it == pl->variant_tw.end() ? nullptr : it->second;
     if (pl->rc.variant >= 0 && !pl->rc.stw) pl->rc.variant = -1;

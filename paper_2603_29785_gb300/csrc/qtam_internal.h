@@ -47,8 +47,29 @@ template <typename T> struct DenseArgs {
   T scale = (T)0;
 };
 
+// One pass of the long FFT over a batch of n-point segments: columns (of length n1,
+// other = n2 of them) or rows (of length n2, other = n1 of them).
+struct LongPass {
+  int n, other;
+  const float2* in;
+  float2* out;
+  const float2* tw4;   // four-step twiddles, [n1][n2]
+  const float2* tws;   // stage twiddles of the length
+};
+using LongFn = cudaError_t (*)(const LongPass&, unsigned batch, cudaStream_t);
+// Kernels of one sub-length (kernels_long_any.cu, FP32); no column pass above 640.
+struct LongShapeFns {
+  int M;
+  int nst, r[kMaxStages];
+  LongFn col_fwd, col_inv, row_fwd, row_inv;
+};
+// the shape of sub-length M, or nullptr: every 2^a 3^b 5^c from 16 to 1296
+const LongShapeFns* long_shape(int M);
+
 // Long real FFT of N = 2n samples as an n = n1 * n2 four-step complex FFT.
 struct LongCfg {
+  const LongShapeFns* cols = nullptr;   // compile-time passes, where they serve (FP32) ...
+  const LongShapeFns* rows = nullptr;   // ... else the engines below
   const void* stw_col = nullptr;   // stage twiddle tables of the static column engine (or null)
   const void* stw_row = nullptr;   // ... of the static row engine
   const void* tw4 = nullptr;       // [n1][n2] four-step twiddles w_n^(k1 c), layout of the column-pass output
