@@ -82,39 +82,47 @@ __global__ void k_scale_rows(typename Env<V, E>::S* __restrict__ y, const float*
 }
 
 // Per (segment, plane) pair: energy = sum |Y|^2 and peak = max |Y|^2 over
-// the K*M envelope values (App. A optimal-plane selection).  Each pair is
-// split over kMetricChunks blocks so the read of Y runs at HBM speed; FP32
-// envelopes are squared in FP32 and summed in FP32 partials of at most 8
-// terms (relative error <= ~5e-7) before FP64 accumulation (the FP64 pipe is
-// slow on this part); FP64 envelopes stay in FP64.  Blocks combine with a
-// double atomicAdd and an integer atomicMax on the (non-negative) float bits;
-// both outputs are zeroed by the launcher first.
-constexpr int kMetricChunks = 64;
+// the K*M envelope values (App. A optimal-plane selection).  FP32 envelopes are
+// squared in FP32 and summed in FP32 partials of at most 8 terms (relative
+// error <= ~5e-7) before FP64 accumulation; FP64 envelopes stay in FP64.  The
+// partials are those of 64 parts a pair, element i of a part in partial
+// (i / 2048, i mod 256), however the parts are spread over blocks: another
+// grouping would move the energies by more than their FP64 sums resolve.
+// Blocks combine with a double atomicAdd and an integer atomicMax on the
+// (non-negative) float bits; both outputs are zeroed by the launcher first.
+//
+// The FP64 pipe (2 lanes a cycle and SM) bounds the reduction, not the read: one
+// block per part spent ten FP64 instructions a warp on two or three elements a
+// thread (128 x 5 planes of 62 x 675: 186 us, 14 % of HBM).  A block now takes
+// `parts` consecutive parts, as many as leave about eight blocks an SM, and
+// reduces once.
+constexpr int kMetricParts = 64;
 
 template <typename V, int E>
-__global__ void __launch_bounds__(256) k_plane_metrics(const typename Env<V, E>::S* __restrict__ y, int64_t per_plane,
+__global__ void __launch_bounds__(256) k_plane_metrics(const typename Env<V, E>::S* __restrict__ y, int64_t per_plane, int parts,
                                                        double* __restrict__ energy, float* __restrict__ peak) {
   using R = decltype(V().x);
-  const int64_t pair = blockIdx.x / kMetricChunks;
-  const int part = (int)(blockIdx.x - pair * kMetricChunks);
-  const int64_t len = (per_plane + kMetricChunks - 1) / kMetricChunks;
-  const int64_t b0 = part * len, b1 = min(per_plane, b0 + len);
+  const int64_t pair = blockIdx.x;
+  const int64_t len = (per_plane + kMetricParts - 1) / kMetricParts;
   const typename Env<V, E>::S* p = y + pair * per_plane;
   double e = 0.0;
   float mx = 0.0f;
-  for (int64_t i0 = b0 + threadIdx.x; i0 < b1; i0 += 8 * (int64_t)blockDim.x) {
-    R es = (R)0;
+  for (int part = blockIdx.y * parts; part < (int)(blockIdx.y + 1) * parts; ++part) {
+    const int64_t b0 = part * len, b1 = min(per_plane, b0 + len);
+    for (int64_t i0 = b0 + threadIdx.x; i0 < b1; i0 += 8 * (int64_t)256) {
+      R es = (R)0;
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int64_t i = i0 + (int64_t)u * blockDim.x;
-      if (i < b1) {
-        const V v = Env<V, E>::from(stream_load(&p[i]));
-        const R a2 = v.x * v.x + v.y * v.y;
-        es += a2;
-        mx = fmaxf(mx, (float)a2);
+      for (int u = 0; u < 8; ++u) {
+        const int64_t i = i0 + u * 256;
+        if (i < b1) {
+          const V v = Env<V, E>::from(stream_load(&p[i]));
+          const R a2 = v.x * v.x + v.y * v.y;
+          es += a2;
+          mx = fmaxf(mx, (float)a2);
+        }
       }
+      e += (double)es;
     }
-    e += (double)es;
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -149,19 +157,22 @@ cudaError_t launch_plane_metrics(const void* y, int env, int64_t pairs, int64_t 
   cudaError_t e0 = cudaMemsetAsync(energy, 0, (size_t)pairs * sizeof(double), st);
   if (e0 == cudaSuccess) e0 = cudaMemsetAsync(peak, 0, (size_t)pairs * sizeof(float), st);
   if (e0 != cudaSuccess) return e0;
-  const unsigned grid = (unsigned)(pairs * kMetricChunks);
+  // a power of two, so that it divides the 64; 1216 = 8 blocks on each of 152 SMs
+  int parts = 1;
+  while (parts < kMetricParts && pairs * (kMetricParts / parts) >= 2 * 1216) parts *= 2;
+  const dim3 grid((unsigned)pairs, (unsigned)(kMetricParts / parts));
   switch (env) {
     case ENV_F64:
-      k_plane_metrics<double2, ENV_F64><<<grid, 256, 0, st>>>(static_cast<const double2*>(y), per_plane, energy, peak);
+      k_plane_metrics<double2, ENV_F64><<<grid, 256, 0, st>>>(static_cast<const double2*>(y), per_plane, parts, energy, peak);
       break;
     case ENV_BF16:
-      k_plane_metrics<float2, ENV_BF16><<<grid, 256, 0, st>>>(static_cast<const __nv_bfloat162*>(y), per_plane, energy, peak);
+      k_plane_metrics<float2, ENV_BF16><<<grid, 256, 0, st>>>(static_cast<const __nv_bfloat162*>(y), per_plane, parts, energy, peak);
       break;
     case ENV_F16:
-      k_plane_metrics<float2, ENV_F16><<<grid, 256, 0, st>>>(static_cast<const __half2*>(y), per_plane, energy, peak);
+      k_plane_metrics<float2, ENV_F16><<<grid, 256, 0, st>>>(static_cast<const __half2*>(y), per_plane, parts, energy, peak);
       break;
     default:
-      k_plane_metrics<float2, ENV_F32><<<grid, 256, 0, st>>>(static_cast<const float2*>(y), per_plane, energy, peak);
+      k_plane_metrics<float2, ENV_F32><<<grid, 256, 0, st>>>(static_cast<const float2*>(y), per_plane, parts, energy, peak);
   }
   return cudaGetLastError();
 }
