@@ -275,6 +275,12 @@ QTAM_API qtam_status qtam_roundtrip_host(qtam_plan_t plan, const void* x_host, i
 QTAM_API qtam_status qtam_plane_metrics(qtam_plan_t plan, const void* y, int64_t batch, double* energy, float* peak,
                                         void* stream);
 
+/* The optimal plane of every segment from those metrics: best_energy[b] and
+ * best_peak[b] (int64) are the first plane with the largest energy and peak of
+ * segment b; a NaN counts as larger than any number. */
+QTAM_API qtam_status qtam_best_planes(qtam_plan_t plan, const double* energy, const float* peak, int64_t batch,
+                             int64_t* best_energy, int64_t* best_peak, void* stream);
+
 /* Multiply every envelope row by a gain: y[b][p][k][*] *= gain[(b*P + p)*K + k]
  * (gain: device float array of batch*P*K entries).  Gain 0 zeroes a row --
  * the masked (row-zeroed) envelopes the inverse accepts; gain 1 leaves the

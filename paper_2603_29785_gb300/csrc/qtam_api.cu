@@ -1298,6 +1298,18 @@ qtam_status qtam_plane_metrics(qtam_plan_t pl, const void* y, int64_t B, double*
   return e == cudaSuccess ? QTAM_OK : fail_cuda(e, "plane_metrics launch");
 }
 
+qtam_status qtam_best_planes(qtam_plan_t pl, const double* energy, const float* peak, int64_t B, int64_t* best_energy,
+                             int64_t* best_peak, void* stream) {
+  qtam_status s = common_checks(pl, B);
+  if (s != QTAM_OK || B == 0) return s;
+  if (!energy || !peak || !best_energy || !best_peak) return fail(QTAM_ERR_INVALID_ARG, "NULL buffer");
+  if (!aligned(energy, 8) || !aligned(peak, 4) || !aligned(best_energy, 8) || !aligned(best_peak, 8))
+    return fail(QTAM_ERR_INVALID_ARG, "misaligned buffer");
+  DeviceGuard g(pl->device);
+  cudaError_t e = launch_best_planes(energy, peak, B, pl->P, best_energy, best_peak, static_cast<cudaStream_t>(stream));
+  return e == cudaSuccess ? QTAM_OK : fail_cuda(e, "best_planes launch");
+}
+
 qtam_status qtam_scale_rows(qtam_plan_t pl, void* y, int64_t B, const float* gain, void* stream) {
   qtam_status s = common_checks(pl, B);
   if (s != QTAM_OK || B == 0) return s;

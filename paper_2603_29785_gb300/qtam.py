@@ -105,6 +105,7 @@ SIGNATURES = {
     "qtam_forward_noalloc": (ctypes.c_int, [_P, _P, _I64, _P, _P]),
     "qtam_scale_rows": (ctypes.c_int, [_P, _P, _I64, _P, _P]),
     "qtam_plane_metrics": (ctypes.c_int, [_P, _P, _I64, _P, _P, _P]),
+    "qtam_best_planes": (ctypes.c_int, [_P, _P, _P, _I64, _P, _P, _P]),
     "qtam_batched_workspace_size": (ctypes.c_int, [_P, ctypes.c_int32, ctypes.POINTER(_SZ)]),
     "qtam_forward_batched": (ctypes.c_int, [_P, ctypes.c_int32, _P, _SZ, _P]),
     "qtam_inverse_batched": (ctypes.c_int, [_P, ctypes.c_int32, _U64, _P, _SZ, _P]),
@@ -312,6 +313,11 @@ def qtam_forward_noalloc(plan, x, batch, y, stream=None):
 
 def qtam_plane_metrics(plan, y, batch, energy, peak, stream=None):
     _check(lib().qtam_plane_metrics(plan, _ptr(y), int(batch), _ptr(energy), _ptr(peak), _stream(stream)))
+
+
+def qtam_best_planes(plan, energy, peak, batch, best_energy, best_peak, stream=None):
+    _check(lib().qtam_best_planes(plan, _ptr(energy), _ptr(peak), int(batch), _ptr(best_energy), _ptr(best_peak),
+                                  _stream(stream)))
 
 
 def qtam_scale_rows(plan, y, batch, gain, stream=None):
@@ -545,8 +551,11 @@ class Plan:
         B = y.shape[0]
         energy = torch.empty((B, self.P), dtype=torch.float64, device=y.device)
         peak = torch.empty((B, self.P), dtype=torch.float32, device=y.device)
+        best_energy = torch.empty((B,), dtype=torch.int64, device=y.device)
+        best_peak = torch.empty((B,), dtype=torch.int64, device=y.device)
         qtam_plane_metrics(self.handle, y, B, energy, peak, stream)
-        return energy, peak, energy.argmax(dim=1), peak.argmax(dim=1)
+        qtam_best_planes(self.handle, energy, peak, B, best_energy, best_peak, stream)
+        return energy, peak, best_energy, best_peak
 
     def scale_rows(self, y, gain, stream=None):
         """y[b, p, k, :] *= gain[b, p, k] in place (gain: CUDA float32 [batch, P, K])."""
