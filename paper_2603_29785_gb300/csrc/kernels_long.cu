@@ -27,7 +27,7 @@ struct GenLong {
   static constexpr int NT = kMaxBlock;
   static constexpr int MINB = 1;
   __device__ __forceinline__ int m() const { return rp.m; }
-  __device__ __forceinline__ int nb_shift() const { return nbs; }
+  __host__ __device__ __forceinline__ int nb_shift() const { return nbs; }
   template <int S, typename V, class L, class St>
   __device__ __forceinline__ void run(V* sm, const V* tw, int twstride, const L& ld, const St& st) const {
     block_fft<S>(rp, nbs, sm, tw, twstride, ld, st);
@@ -41,7 +41,7 @@ template <int M_, int NBS_, int NT_, int... Rs> struct StatLong {
   static constexpr int NT = NT_ > 0 ? NT_ : StaticThreads<M_, NBS_, Rs...>::value;
   static constexpr int MINB = NT >= 512 ? 1 : 512 / NT;   // at least 512 threads per SM
   __device__ __forceinline__ int m() const { return M_; }
-  __device__ __forceinline__ int nb_shift() const { return NBS_; }
+  __host__ __device__ __forceinline__ int nb_shift() const { return NBS_; }
   template <int S, typename V, class L, class St>
   __device__ __forceinline__ void run(V* sm, const V* tws, int, const L& ld, const St& st) const {
     StaticFFT<S, M_, NT, NBS_, Rs...>::run(sm, tws, ld, st);
@@ -105,7 +105,13 @@ template <typename V> __device__ __forceinline__ V wN(const V* twN, int n, int k
   return mk<V>(-t.x, t.y);
 }
 
-constexpr int kUntanglePairs = 4;   // (k, n-k) pairs per thread, for memory-level parallelism
+// (k, n-k) pairs a thread and threads a block.  FP32: four, for memory-level
+// parallelism.  FP64: one, in small blocks, because the FP64 pipe (2 lanes a cycle and
+// SM) bounds it and 1024 pairs a block left all but five SMs idle at n = 8192 (8.4 us).
+template <typename T> struct Untangle {
+  static constexpr int PAIRS = sizeof(T) == 8 ? 1 : 4, NT = sizeof(T) == 8 ? 64 : 256;
+  static dim3 grid(int n, int64_t nb) { return dim3((unsigned)((n / 2 + 1 + NT * PAIRS - 1) / (NT * PAIRS)), (unsigned)nb); }
+};
 
 template <typename T>
 __global__ void k_untangle_forward(int n, const cplx<T>* __restrict__ Z, cplx<T>* __restrict__ X,
@@ -115,9 +121,9 @@ __global__ void k_untangle_forward(int n, const cplx<T>* __restrict__ Z, cplx<T>
   const V* Zs = Z + seg * n;
   V* Xs = X + seg * (int64_t)(n + 1);
   const T half = (T)0.5;
-  const int base = blockIdx.x * blockDim.x * kUntanglePairs + threadIdx.x;
+  const int base = blockIdx.x * blockDim.x * Untangle<T>::PAIRS + threadIdx.x;
 #pragma unroll
-  for (int u = 0; u < kUntanglePairs; ++u) {
+  for (int u = 0; u < Untangle<T>::PAIRS; ++u) {
     const int k = base + u * blockDim.x;
     if (k > (n >> 1)) break;
     const int kk = n - k;                     // partner bin, in [n/2, n]
@@ -159,9 +165,9 @@ __global__ void k_untangle_inverse(int n, const cplx<T>* __restrict__ A, const T
   const V* As = A + seg * (int64_t)(n + 1);
   V* Zs = Zi + seg * n;
   const T hs = (T)0.5 * scale;
-  const int base = blockIdx.x * blockDim.x * kUntanglePairs + threadIdx.x;
+  const int base = blockIdx.x * blockDim.x * Untangle<T>::PAIRS + threadIdx.x;
 #pragma unroll
-  for (int u = 0; u < kUntanglePairs; ++u) {
+  for (int u = 0; u < Untangle<T>::PAIRS; ++u) {
     const int k = base + u * blockDim.x;
     if (k > (n >> 1)) break;
     const int kk = n - k;                     // in [n/2, n]
@@ -234,10 +240,19 @@ constexpr int64_t kMaxGridY = 65535;
   X(512, NBS, (NBS == 2 ? 64 : 0), 16, 32)     \
   X(1024, NBS, 0, 32, 32)
 
+template <class Eng> unsigned pass_threads(const Eng&) { return Eng::NT; }
+// The runtime engine runs a stage's items in rounds over whatever threads there are.
+unsigned pass_threads(const GenLong& eng) { return (unsigned)spread_threads(eng.rp, eng.nbs); }
 template <class Eng, class K, class... Args>
 void launch_pass(K kernel, const Eng& eng, size_t smem, dim3 g, cudaStream_t st, Args... args) {
   allow_smem((const void*)kernel, smem);
-  kernel<<<g, Eng::NT, smem, st>>>(eng, args...);
+  kernel<<<g, pass_threads(eng), smem, st>>>(eng, args...);
+}
+// Transforms per block of a runtime pass over `count` of them: as many as the plan
+// allows for coalescing, fewer while the grid leaves SMs without a block.
+int gen_nbs(int nbs, int64_t count, int64_t batch) {
+  while (nbs > 0 && (count >> nbs) * batch < 2 * 152) --nbs;
+  return nbs;
 }
 
 // Call f(engine, smem) with the static engine for (m, nbs) when one exists
@@ -254,7 +269,7 @@ void launch_pass(K kernel, const Eng& eng, size_t smem, dim3 g, cudaStream_t st,
 // runtime engine with the plan's length-n table.
 template <typename T, class F>
 void with_engine(const RadixPlan& rp, int nbs, int static_nbs, size_t gen_smem, const void* stw,
-                 const cplx<T>* twn, F&& f) {
+                 const cplx<T>* twn, int count, int64_t batch, F&& f) {
   if constexpr (sizeof(T) == 4) {
     if (stw && nbs == static_nbs && static_nbs == 4) {
       switch (rp.m) { QTAM_LONG_CASES(QTAM_CASE, 4) default: break; }
@@ -262,7 +277,7 @@ void with_engine(const RadixPlan& rp, int nbs, int static_nbs, size_t gen_smem, 
       switch (rp.m) { QTAM_LONG_CASES(QTAM_CASE, 2) default: break; }
     }
   }
-  f(GenLong{rp, nbs}, gen_smem, twn);
+  f(GenLong{rp, gen_nbs(nbs, count, batch)}, gen_smem, twn);
 }
 #undef QTAM_CASE
 
@@ -328,9 +343,9 @@ cudaError_t launch_spectrum(const LongCfg& c, const cplx<T>* z, cplx<T>* U, cplx
       const cudaError_t e = launch_shape<T>(c.cols->col_fwd, c, true, z + off, U + off, nb, st);
       if (e != cudaSuccess) return e;
     } else {
-      with_engine<T>(c.rp1, c.col_nbs, 4, c.col_smem, c.stw_col, twn, [&](auto eng, size_t smem, const cplx<T>* ftw) {
+      with_engine<T>(c.rp1, c.col_nbs, 4, c.col_smem, c.stw_col, twn, c.n2, nb, [&](auto eng, size_t smem, const cplx<T>* ftw) {
         using E = decltype(eng);
-        dim3 g(c.n2 >> c.col_nbs, (unsigned)nb);
+        dim3 g(c.n2 >> eng.nb_shift(), (unsigned)nb);
         launch_pass(k_col_forward<E, T>, eng, smem, g, st, c.n, c.n2, z + off, U + off, tw4, ftw);
       });
     }
@@ -338,14 +353,13 @@ cudaError_t launch_spectrum(const LongCfg& c, const cplx<T>* z, cplx<T>* U, cplx
       const cudaError_t e = launch_shape<T>(c.rows->row_fwd, c, false, (const cplx<T>*)(U + off), Z + off, nb, st);
       if (e != cudaSuccess) return e;
     } else {
-      with_engine<T>(c.rp2, c.row_nbs, 2, c.row_smem, c.stw_row, twn, [&](auto eng, size_t smem, const cplx<T>* ftw) {
+      with_engine<T>(c.rp2, c.row_nbs, 2, c.row_smem, c.stw_row, twn, c.n1, nb, [&](auto eng, size_t smem, const cplx<T>* ftw) {
         using E = decltype(eng);
-        dim3 g(c.n1 >> c.row_nbs, (unsigned)nb);
+        dim3 g(c.n1 >> eng.nb_shift(), (unsigned)nb);
         launch_pass(k_row_forward<E, T>, eng, smem, g, st, c.n, c.n1, (const cplx<T>*)(U + off), Z + off, ftw);
       });
     }
-    dim3 g3((unsigned)((c.n / 2 + 1 + 256 * kUntanglePairs - 1) / (256 * kUntanglePairs)), (unsigned)nb);
-    k_untangle_forward<T><<<g3, 256, 0, st>>>(c.n, Z + off, X + s0 * (int64_t)(c.n + 1), twN);
+    k_untangle_forward<T><<<Untangle<T>::grid(c.n, nb), Untangle<T>::NT, 0, st>>>(c.n, Z + off, X + s0 * (int64_t)(c.n + 1), twN);
   }
   return cudaGetLastError();
 }
@@ -357,16 +371,15 @@ cudaError_t launch_synthesis(const LongCfg& c, const cplx<T>* A, const T* invP, 
   for (int64_t s0 = 0; s0 < B; s0 += kMaxGridY) {
     const int64_t nb = (B - s0) < kMaxGridY ? (B - s0) : kMaxGridY;
     const int64_t off = s0 * c.n;
-    dim3 g0((unsigned)((c.n / 2 + 1 + 256 * kUntanglePairs - 1) / (256 * kUntanglePairs)), (unsigned)nb);
-    k_untangle_inverse<T><<<g0, 256, 0, st>>>(c.n, A + s0 * (int64_t)(c.n + 1), invP, Zi + off, twN,
+    k_untangle_inverse<T><<<Untangle<T>::grid(c.n, nb), Untangle<T>::NT, 0, st>>>(c.n, A + s0 * (int64_t)(c.n + 1), invP, Zi + off, twN,
                                               (T)1 / (T)c.n);
     if (c.rows) {
       const cudaError_t e = launch_shape<T>(c.rows->row_inv, c, false, (const cplx<T>*)(Zi + off), Vb + off, nb, st);
       if (e != cudaSuccess) return e;
     } else {
-      with_engine<T>(c.rp2, c.row_nbs, 2, c.row_smem, c.stw_row, twn, [&](auto eng, size_t smem, const cplx<T>* ftw) {
+      with_engine<T>(c.rp2, c.row_nbs, 2, c.row_smem, c.stw_row, twn, c.n1, nb, [&](auto eng, size_t smem, const cplx<T>* ftw) {
         using E = decltype(eng);
-        dim3 g(c.n1 >> c.row_nbs, (unsigned)nb);
+        dim3 g(c.n1 >> eng.nb_shift(), (unsigned)nb);
         launch_pass(k_row_inverse<E, T>, eng, smem, g, st, c.n, c.n1, (const cplx<T>*)(Zi + off), Vb + off, tw4, ftw);
       });
     }
@@ -374,9 +387,9 @@ cudaError_t launch_synthesis(const LongCfg& c, const cplx<T>* A, const T* invP, 
       const cudaError_t e = launch_shape<T>(c.cols->col_inv, c, true, (const cplx<T>*)(Vb + off), xout + off, nb, st);
       if (e != cudaSuccess) return e;
     } else {
-      with_engine<T>(c.rp1, c.col_nbs, 4, c.col_smem, c.stw_col, twn, [&](auto eng, size_t smem, const cplx<T>* ftw) {
+      with_engine<T>(c.rp1, c.col_nbs, 4, c.col_smem, c.stw_col, twn, c.n2, nb, [&](auto eng, size_t smem, const cplx<T>* ftw) {
         using E = decltype(eng);
-        dim3 g(c.n2 >> c.col_nbs, (unsigned)nb);
+        dim3 g(c.n2 >> eng.nb_shift(), (unsigned)nb);
         launch_pass(k_col_inverse<E, T>, eng, smem, g, st, c.n, c.n2, (const cplx<T>*)(Vb + off), xout + off, ftw);
       });
     }

@@ -245,6 +245,18 @@ cudaError_t launch_best_planes(const double* energy, const float* peak, int64_t 
 cudaError_t launch_scale_rows(void* y, int env, const float* gain, int64_t n_rows, int M, cudaStream_t st);
 const RowVariant* row_variant(int i);   // nullptr when out of range
 
+// Threads for the runtime engine: one per item of the stage with the most items, so
+// that no thread runs rounds while others idle, at most a block's 512 (the rounds a
+// thread must then take are within ipt_for: the plan checked threads_for <= 512).
+inline int spread_threads(const RadixPlan& rp, int nbs) {
+  int t = 32;
+  for (int s = 0; s < rp.nst; ++s) {
+    const int items = (rp.m / rp.r[s]) << nbs;
+    t = items > t ? items : t;
+  }
+  return t > kMaxBlock ? kMaxBlock : (t + 31) / 32 * 32;
+}
+
 // ---- launchers (kernels_long.cu) ----
 // z: [B][n] complex view of the real input; U: [B][n]; Z: [B][n]; X: [B][n+1]
 template <typename T>

@@ -51,3 +51,11 @@ def check(N, compute, tol):
 def test_lengths_f32(group):
     for n in HALVES[group::GROUPS]:
         check(2 * n, "f32", 1e-6)
+
+
+@pytest.mark.parametrize("group", range(4))
+def test_lengths_f64(group):
+    """Every eighth length in FP64: 1.1e-16 sqrt(log2 N) <= 5e-16 a transform, tables as much again, FP64
+    reference alike; 1e-14 leaves a factor of five."""
+    for n in HALVES[2 * group::32]:
+        check(2 * n, "f64", 1e-14)
