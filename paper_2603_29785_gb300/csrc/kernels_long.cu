@@ -33,20 +33,20 @@ struct GenLong {
     block_fft<S>(rp, nbs, sm, tw, twstride, ld, st);
   }
 };
-// NT_ = 0: the block spans the widest stage's items; otherwise NT_ threads and
-// wider stages run in rounds
-template <int M_, int NBS_, int NT_, int... Rs> struct StatLong {
+constexpr int kLongColsLog2 = 4;   // columns a block of the static column engines, log2
+template <int M_, int... Rs> struct StatLong {
+  static constexpr int NBS = kLongColsLog2;
   static constexpr int nrad = sizeof...(Rs);
   static constexpr int radices[nrad] = {Rs...};
-  static constexpr int NT = NT_ > 0 ? NT_ : StaticThreads<M_, NBS_, Rs...>::value;
-  static constexpr int MINB = NT >= 512 ? 1 : 512 / NT;   // at least 512 threads per SM
+  static constexpr int NT = StaticThreads<M_, NBS, Rs...>::value;   // the widest stage's items
+  static constexpr int MINB = NT >= 512 ? 1 : 512 / NT;             // at least 512 threads per SM
   __device__ __forceinline__ int m() const { return M_; }
-  __host__ __device__ __forceinline__ int nb_shift() const { return NBS_; }
+  __host__ __device__ __forceinline__ int nb_shift() const { return NBS; }
   template <int S, typename V, class L, class St>
   __device__ __forceinline__ void run(V* sm, const V* tws, int, const L& ld, const St& st) const {
-    StaticFFT<S, M_, NT, NBS_, Rs...>::run(sm, tws, ld, st);
+    StaticFFT<S, M_, NT, NBS, Rs...>::run(sm, tws, ld, st);
   }
-  static size_t smem_bytes(size_t elem) { return StaticFFT<1, M_, NT, NBS_, Rs...>::smem_elems() * elem; }
+  static size_t smem_bytes(size_t elem) { return StaticFFT<1, M_, NT, NBS, Rs...>::smem_elems() * elem; }
 };
 
 template <typename V> struct LoadColumns {
@@ -227,18 +227,17 @@ __global__ void __launch_bounds__(Eng::NT, Eng::MINB) k_col_inverse(Eng eng, int
 
 constexpr int64_t kMaxGridY = 65535;
 
-// Static engines for power-of-two sub-lengths (FP32): column passes
-// interleave 16 columns, row passes 4 rows.  The 512-point row pass runs on
-// 64 threads (its 16-point stage in two rounds) rather than 128, of which
-// the 32-point stage kept half idle: the 64 s spectrum 0.0897 -> 0.0856 ms,
-// the synthesis 0.0948 -> 0.0938 ms per 64 segments.
-#define QTAM_LONG_CASES(X, NBS)                \
-  X(32, NBS, 0, 8, 4)                          \
-  X(64, NBS, 0, 16, 4)                         \
-  X(128, NBS, 0, 16, 8)                        \
-  X(256, NBS, 0, 16, 16)                       \
-  X(512, NBS, (NBS == 2 ? 64 : 0), 16, 32)     \
-  X(1024, NBS, 0, 32, 32)
+// Static engines of the column pass at power-of-two lengths (FP32), 16 columns
+// interleaved: 29.4 and 22.5 us forward and inverse for 64 segments of 131072
+// points, where the pass engine (kernels_long_any.cu), whose exchange is padded for
+// rows, takes 33.4 and 22.6.  Rows of every length run on the pass engine.
+#define QTAM_LONG_CASES(X) \
+  X(32, 8, 4)              \
+  X(64, 16, 4)             \
+  X(128, 16, 8)            \
+  X(256, 16, 16)           \
+  X(512, 16, 32)           \
+  X(1024, 32, 32)
 
 template <class Eng> unsigned pass_threads(const Eng&) { return Eng::NT; }
 // The runtime engine runs a stage's items in rounds over whatever threads there are.
@@ -255,38 +254,33 @@ int gen_nbs(int nbs, int64_t count, int64_t batch) {
   return nbs;
 }
 
-// Call f(engine, smem) with the static engine for (m, nbs) when one exists
-// (FP32), else with the runtime engine.
-#define QTAM_CASE(M, NBS, ...)                                     \
-  case M: {                                                        \
-    using E = StatLong<M, NBS, __VA_ARGS__>;                       \
-    f(E(), E::smem_bytes(sizeof(float2)), (const cplx<T>*)stw);    \
-    return;                                                        \
+#define QTAM_CASE(M, ...)                                       \
+  case M: {                                                     \
+    using E = StatLong<M, __VA_ARGS__>;                         \
+    f(E(), E::smem_bytes(sizeof(float2)), (const cplx<T>*)stw); \
+    return;                                                     \
   }
 
-// Call f(engine, smem bytes, engine twiddles): the static engine for
-// (m, nbs) when one exists (FP32) and its tables were built, else the
-// runtime engine with the plan's length-n table.
+// Call f(engine, smem bytes, engine twiddles): the static column engine where the
+// plan built its tables (stw), else the runtime engine with the length-n table.
 template <typename T, class F>
-void with_engine(const RadixPlan& rp, int nbs, int static_nbs, size_t gen_smem, const void* stw,
-                 const cplx<T>* twn, int count, int64_t batch, F&& f) {
+void with_engine(const RadixPlan& rp, int nbs, size_t gen_smem, const void* stw, const cplx<T>* twn, int count, int64_t batch,
+                 F&& f) {
   if constexpr (sizeof(T) == 4) {
-    if (stw && nbs == static_nbs && static_nbs == 4) {
-      switch (rp.m) { QTAM_LONG_CASES(QTAM_CASE, 4) default: break; }
-    } else if (stw && nbs == static_nbs && static_nbs == 2) {
-      switch (rp.m) { QTAM_LONG_CASES(QTAM_CASE, 2) default: break; }
+    if (stw) {
+      switch (rp.m) { QTAM_LONG_CASES(QTAM_CASE) default: break; }
     }
   }
   f(GenLong{rp, gen_nbs(nbs, count, batch)}, gen_smem, twn);
 }
 #undef QTAM_CASE
 
-#define QTAM_RADICES(M, NBS, ...)                   \
-  case M: {                                         \
-    using E = StatLong<M, NBS, __VA_ARGS__>;        \
-    *nst = E::nrad;                                 \
+#define QTAM_RADICES(M, ...)                                \
+  case M: {                                                 \
+    using E = StatLong<M, __VA_ARGS__>;                     \
+    *nst = E::nrad;                                         \
     for (int i = 0; i < E::nrad; ++i) r[i] = E::radices[i]; \
-    return true;                                    \
+    return true;                                            \
   }
 
 // one pass of a batch through its compile-time shape
@@ -323,11 +317,8 @@ const LongShapeFns* long_shape(int M) {
 #undef QTAM_PARTS
 
 bool long_static_radices(int m, int nbs, int* r, int* nst) {
-  if (nbs == 4) {
-    switch (m) { QTAM_LONG_CASES(QTAM_RADICES, 4) default: break; }
-  } else if (nbs == 2) {
-    switch (m) { QTAM_LONG_CASES(QTAM_RADICES, 2) default: break; }
-  }
+  if (nbs != kLongColsLog2) return false;
+  switch (m) { QTAM_LONG_CASES(QTAM_RADICES) default: break; }
   return false;
 }
 #undef QTAM_RADICES
@@ -343,7 +334,7 @@ cudaError_t launch_spectrum(const LongCfg& c, const cplx<T>* z, cplx<T>* U, cplx
       const cudaError_t e = launch_shape<T>(c.cols->col_fwd, c, true, z + off, U + off, nb, st);
       if (e != cudaSuccess) return e;
     } else {
-      with_engine<T>(c.rp1, c.col_nbs, 4, c.col_smem, c.stw_col, twn, c.n2, nb, [&](auto eng, size_t smem, const cplx<T>* ftw) {
+      with_engine<T>(c.rp1, c.col_nbs, c.col_smem, c.stw_col, twn, c.n2, nb, [&](auto eng, size_t smem, const cplx<T>* ftw) {
         using E = decltype(eng);
         dim3 g(c.n2 >> eng.nb_shift(), (unsigned)nb);
         launch_pass(k_col_forward<E, T>, eng, smem, g, st, c.n, c.n2, z + off, U + off, tw4, ftw);
@@ -353,7 +344,7 @@ cudaError_t launch_spectrum(const LongCfg& c, const cplx<T>* z, cplx<T>* U, cplx
       const cudaError_t e = launch_shape<T>(c.rows->row_fwd, c, false, (const cplx<T>*)(U + off), Z + off, nb, st);
       if (e != cudaSuccess) return e;
     } else {
-      with_engine<T>(c.rp2, c.row_nbs, 2, c.row_smem, c.stw_row, twn, c.n1, nb, [&](auto eng, size_t smem, const cplx<T>* ftw) {
+      with_engine<T>(c.rp2, c.row_nbs, c.row_smem, nullptr, twn, c.n1, nb, [&](auto eng, size_t smem, const cplx<T>* ftw) {
         using E = decltype(eng);
         dim3 g(c.n1 >> eng.nb_shift(), (unsigned)nb);
         launch_pass(k_row_forward<E, T>, eng, smem, g, st, c.n, c.n1, (const cplx<T>*)(U + off), Z + off, ftw);
@@ -377,7 +368,7 @@ cudaError_t launch_synthesis(const LongCfg& c, const cplx<T>* A, const T* invP, 
       const cudaError_t e = launch_shape<T>(c.rows->row_inv, c, false, (const cplx<T>*)(Zi + off), Vb + off, nb, st);
       if (e != cudaSuccess) return e;
     } else {
-      with_engine<T>(c.rp2, c.row_nbs, 2, c.row_smem, c.stw_row, twn, c.n1, nb, [&](auto eng, size_t smem, const cplx<T>* ftw) {
+      with_engine<T>(c.rp2, c.row_nbs, c.row_smem, nullptr, twn, c.n1, nb, [&](auto eng, size_t smem, const cplx<T>* ftw) {
         using E = decltype(eng);
         dim3 g(c.n1 >> eng.nb_shift(), (unsigned)nb);
         launch_pass(k_row_inverse<E, T>, eng, smem, g, st, c.n, c.n1, (const cplx<T>*)(Zi + off), Vb + off, tw4, ftw);
@@ -387,7 +378,7 @@ cudaError_t launch_synthesis(const LongCfg& c, const cplx<T>* A, const T* invP, 
       const cudaError_t e = launch_shape<T>(c.cols->col_inv, c, true, (const cplx<T>*)(Vb + off), xout + off, nb, st);
       if (e != cudaSuccess) return e;
     } else {
-      with_engine<T>(c.rp1, c.col_nbs, 4, c.col_smem, c.stw_col, twn, c.n2, nb, [&](auto eng, size_t smem, const cplx<T>* ftw) {
+      with_engine<T>(c.rp1, c.col_nbs, c.col_smem, c.stw_col, twn, c.n2, nb, [&](auto eng, size_t smem, const cplx<T>* ftw) {
         using E = decltype(eng);
         dim3 g(c.n2 >> eng.nb_shift(), (unsigned)nb);
         launch_pass(k_col_inverse<E, T>, eng, smem, g, st, c.n, c.n2, (const cplx<T>*)(Vb + off), xout + off, ftw);

@@ -512,7 +512,7 @@ template <typename T> qtam_status upload_tables(qtam_plan_s* pl) {
       if ((s = upload_stage_table(rv->r, rv->nst, &p, tot, rv->tw_pair != 0)) != QTAM_OK) return s;
       pl->variant_tw[v] = p;
     }
-    // the passes of the long FFT: powers of two have their own engines
+    // the passes of the long FFT: columns of a power of two have their own engines
     int r[kMaxStages], nst = 0;
     const LongShapeFns* ls = long_shape(pl->lc.n1);
     if (long_static_radices(pl->lc.n1, pl->lc.col_nbs, r, &nst)) {
@@ -522,9 +522,7 @@ template <typename T> qtam_status upload_tables(qtam_plan_s* pl) {
       pl->lc.cols = ls;
     }
     pl->lc.stw_col = pl->d_stw_col;
-    if (long_static_radices(pl->lc.n2, pl->lc.row_nbs, r, &nst)) {
-      if ((s = upload_stage_table(r, nst, &pl->d_stw_row, tot)) != QTAM_OK) return s;
-    } else if ((ls = long_shape(pl->lc.n2))) {
+    if ((ls = long_shape(pl->lc.n2))) {
       if ((s = upload_stage_table(ls->r, ls->nst, &pl->d_stw_row, tot)) != QTAM_OK) return s;
       pl->lc.rows = ls;
     }

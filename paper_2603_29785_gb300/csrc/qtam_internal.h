@@ -70,8 +70,8 @@ const LongShapeFns* long_shape(int M);
 struct LongCfg {
   const LongShapeFns* cols = nullptr;   // compile-time passes, where they serve (FP32) ...
   const LongShapeFns* rows = nullptr;   // ... else the engines below
-  const void* stw_col = nullptr;   // stage twiddle tables of the static column engine (or null)
-  const void* stw_row = nullptr;   // ... of the static row engine
+  const void* stw_col = nullptr;   // stage twiddle tables of the compile-time column pass (or null)
+  const void* stw_row = nullptr;   // ... and row pass
   const void* tw4 = nullptr;       // [n1][n2] four-step twiddles w_n^(k1 c), layout of the column-pass output
   int n;        // N / 2
   int n1, n2;   // column length n1 (stride n2), row length n2
@@ -290,8 +290,8 @@ cudaError_t launch_rows_stream_inverse(const RowCfg& c, const RowDev<float>* row
                                        int n_rows, int64_t Nr, const float2* hist, int hcols, const float2* ynew,
                                        int64_t pitch, int Hn, const float2* phase, float2* A, int64_t B, cudaStream_t st);
 
-// radix sequence of the static long-FFT engine used for a pass of length m
-// with 2^nbs interleaved transforms (FP32); false when the runtime engine runs
+// radix sequence of the static engine of a column pass of length m over blocks of
+// 2^nbs columns (FP32); false when there is none
 bool long_static_radices(int m, int nbs, int* r, int* nst);
 
 // Stage twiddle tables of a compile-time radix sequence r[0..nst), stage 0
