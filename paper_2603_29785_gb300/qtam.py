@@ -126,6 +126,8 @@ SIGNATURES = {
 def lib(build_if_missing: bool = True) -> ctypes.CDLL:
     """Load libqtam.so (building it in-tree first if it is absent or stale)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             path = _build.lib_path()
@@ -143,25 +145,31 @@ def lib(build_if_missing: bool = True) -> ctypes.CDLL:
 
 
 def _check(status: int):
-    if status != QTAM_OK:
+    if status:
         raise QtamError(status, lib().qtam_last_error().decode())
 
 
 def _ptr(t) -> int | None:
-    if t is None:
-        return None
-    if isinstance(t, int):
-        return t
     if hasattr(t, "data_ptr"):
         return t.data_ptr()
+    if t is None or isinstance(t, int):
+        return t
     if isinstance(t, np.ndarray):
         return t.ctypes.data
     raise TypeError(f"cannot pass {type(t)} as a pointer")
 
 
+try:
+    from torch._C import _cuda_getCurrentRawStream as _raw_stream
+except ImportError:        # host-only PyTorch, or none
+    _raw_stream = None
+
+
 def _stream(stream) -> int | None:
     if stream is None:
         import torch
+        if _raw_stream is not None and torch.cuda.is_initialized():
+            return _raw_stream(torch.cuda.current_device())    # without a Stream object per call
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
@@ -405,9 +413,12 @@ def qtam_status_string(status: int) -> str:
 def _require(t, shape, dtypes, device, name):
     """Reject a tensor whose shape, dtype, device or layout does not match
     what the C entry point will read or write (the ABI sees raw pointers)."""
-    ok = (hasattr(t, "is_cuda") and t.is_cuda and t.device.index == device and t.dtype in dtypes
-          and t.is_contiguous() and t.dim() == len(shape)
-          and all(s is None or int(d) == s for d, s in zip(t.shape, shape)))
+    ok = (hasattr(t, "is_cuda") and t.is_cuda and t.get_device() == device and t.dtype in dtypes
+          and t.is_contiguous() and t.dim() == len(shape))
+    if ok:
+        for d, s in zip(t.shape, shape):
+            if s is not None and d != s:
+                ok = False
     if not ok:
         want = "[" + ", ".join("batch" if s is None else str(s) for s in shape) + "]"
         got = (tuple(t.shape), getattr(t, "dtype", None), getattr(t, "device", None)) if hasattr(t, "shape") else type(t)
@@ -453,6 +464,7 @@ class Plan:
         shp = (self.P, self.K)
         self.geometry = Geometry(r["f"].reshape(shp), r["kc"].reshape(shp), r["h"].reshape(shp), r["c"].reshape(shp))
         self._ws = {}
+        self._need = (-1, 0)     # workspace bytes of the last batch size asked for
 
     def __del__(self):
         try:
@@ -466,7 +478,10 @@ class Plan:
 
     def workspace(self, batch: int):
         import torch
-        need = qtam_workspace_size(self.handle, batch)
+        last, need = self._need
+        if last != batch:
+            need = qtam_workspace_size(self.handle, batch)
+            self._need = (batch, need)
         ws = self._ws.get(self.device)
         if ws is None or ws.numel() < need:
             ws = torch.empty(max(need, 256), dtype=torch.uint8, device=f"cuda:{self.device}")
