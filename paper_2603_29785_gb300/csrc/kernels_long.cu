@@ -78,6 +78,7 @@ __global__ void __launch_bounds__(Eng::NT, Eng::MINB) k_col_forward(Eng eng, int
   using V = cplx<T>;
   extern __shared__ __align__(16) unsigned char smraw[];
   V* sm = reinterpret_cast<V*>(smraw);
+  after_previous();
   const int64_t seg = blockIdx.y;
   const int c0 = blockIdx.x << eng.nb_shift();
   LoadColumns<V> ld{z + seg * n, n2, c0};
@@ -91,6 +92,7 @@ __global__ void __launch_bounds__(Eng::NT, Eng::MINB) k_row_forward(Eng eng, int
   using V = cplx<T>;
   extern __shared__ __align__(16) unsigned char smraw[];
   V* sm = reinterpret_cast<V*>(smraw);
+  after_previous();
   const int64_t seg = blockIdx.y;
   const int r0 = blockIdx.x << eng.nb_shift();
   LoadRows<V> ld{U + seg * n, eng.m(), r0};
@@ -117,6 +119,7 @@ template <typename T>
 __global__ void k_untangle_forward(int n, const cplx<T>* __restrict__ Z, cplx<T>* __restrict__ X,
                                    const cplx<T>* __restrict__ twN) {
   using V = cplx<T>;
+  after_previous();
   const int64_t seg = blockIdx.y;
   const V* Zs = Z + seg * n;
   V* Xs = X + seg * (int64_t)(n + 1);
@@ -161,6 +164,7 @@ template <typename T>
 __global__ void k_untangle_inverse(int n, const cplx<T>* __restrict__ A, const T* __restrict__ invP,
                                    cplx<T>* __restrict__ Zi, const cplx<T>* __restrict__ twN, T scale) {
   using V = cplx<T>;
+  after_previous();
   const int64_t seg = blockIdx.y;
   const V* As = A + seg * (int64_t)(n + 1);
   V* Zs = Zi + seg * n;
@@ -205,6 +209,7 @@ __global__ void __launch_bounds__(Eng::NT, Eng::MINB) k_row_inverse(Eng eng, int
   using V = cplx<T>;
   extern __shared__ __align__(16) unsigned char smraw[];
   V* sm = reinterpret_cast<V*>(smraw);
+  after_previous();
   const int64_t seg = blockIdx.y;
   const int r0 = blockIdx.x << eng.nb_shift();
   LoadRowsTransposed<V> ld{Zi + seg * n, n1, r0};
@@ -218,6 +223,7 @@ __global__ void __launch_bounds__(Eng::NT, Eng::MINB) k_col_inverse(Eng eng, int
   using V = cplx<T>;
   extern __shared__ __align__(16) unsigned char smraw[];
   V* sm = reinterpret_cast<V*>(smraw);
+  after_previous();
   const int64_t seg = blockIdx.y;
   const int c0 = blockIdx.x << eng.nb_shift();
   LoadColumns<V> ld{Vb + seg * n, n2, c0};
@@ -243,9 +249,9 @@ template <class Eng> unsigned pass_threads(const Eng&) { return Eng::NT; }
 // The runtime engine runs a stage's items in rounds over whatever threads there are.
 unsigned pass_threads(const GenLong& eng) { return (unsigned)spread_threads(eng.rp, eng.nbs); }
 template <class Eng, class K, class... Args>
-void launch_pass(K kernel, const Eng& eng, size_t smem, dim3 g, cudaStream_t st, Args... args) {
-  allow_smem((const void*)kernel, smem);
-  kernel<<<g, pass_threads(eng), smem, st>>>(eng, args...);
+cudaError_t launch_pass(K kernel, const Eng& eng, size_t smem, dim3 g, cudaStream_t st, Args... args) {
+  const cudaError_t e = allow_smem((const void*)kernel, smem);
+  return e == cudaSuccess ? launch_next(kernel, g, pass_threads(eng), smem, st, eng, args...) : e;
 }
 // Transforms per block of a runtime pass over `count` of them: as many as the plan
 // allows for coalescing, fewer while the grid leaves SMs without a block.
@@ -350,7 +356,9 @@ cudaError_t launch_spectrum(const LongCfg& c, const cplx<T>* z, cplx<T>* U, cplx
         launch_pass(k_row_forward<E, T>, eng, smem, g, st, c.n, c.n1, (const cplx<T>*)(U + off), Z + off, ftw);
       });
     }
-    k_untangle_forward<T><<<Untangle<T>::grid(c.n, nb), Untangle<T>::NT, 0, st>>>(c.n, Z + off, X + s0 * (int64_t)(c.n + 1), twN);
+    const cudaError_t e = launch_next(k_untangle_forward<T>, Untangle<T>::grid(c.n, nb), Untangle<T>::NT, 0, st, c.n, Z + off,
+                                      X + s0 * (int64_t)(c.n + 1), twN);
+    if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
 }
@@ -362,8 +370,9 @@ cudaError_t launch_synthesis(const LongCfg& c, const cplx<T>* A, const T* invP, 
   for (int64_t s0 = 0; s0 < B; s0 += kMaxGridY) {
     const int64_t nb = (B - s0) < kMaxGridY ? (B - s0) : kMaxGridY;
     const int64_t off = s0 * c.n;
-    k_untangle_inverse<T><<<Untangle<T>::grid(c.n, nb), Untangle<T>::NT, 0, st>>>(c.n, A + s0 * (int64_t)(c.n + 1), invP, Zi + off, twN,
-                                              (T)1 / (T)c.n);
+    const cudaError_t e0 = launch_next(k_untangle_inverse<T>, Untangle<T>::grid(c.n, nb), Untangle<T>::NT, 0, st, c.n,
+                                       A + s0 * (int64_t)(c.n + 1), invP, Zi + off, twN, (T)1 / (T)c.n);
+    if (e0 != cudaSuccess) return e0;
     if (c.rows) {
       const cudaError_t e = launch_shape<T>(c.rows->row_inv, c, false, (const cplx<T>*)(Zi + off), Vb + off, nb, st);
       if (e != cudaSuccess) return e;

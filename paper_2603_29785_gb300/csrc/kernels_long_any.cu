@@ -44,6 +44,7 @@ __global__ void __launch_bounds__(Sh::NT, Sh::MINB) k_long_columns(const __grid_
   float2* out = g.out + seg + c0;
   const float2* tw4 = g.tw4 + c0;
   const int cols = n2 - c0;
+  after_previous();
   auto ld = [&](int b, int j, float2* a) {
     if (b < cols) {
       const float2* p = in + (int64_t)j * n2 + b;
@@ -75,6 +76,7 @@ __global__ void __launch_bounds__(Sh::NT, Sh::MINB) k_long_rows(const __grid_con
   const int64_t seg = (int64_t)blockIdx.y * g.n;
   const int r0 = blockIdx.x * NB, n1 = g.other;
   const int rows = n1 - r0;
+  after_previous();
   // natural: row r0 + b of [n1][M]; transposed: column r0 + b of [M][n1]
   auto ld = [&](int b, int j, float2* a) {
     if (b < rows) {
@@ -115,8 +117,7 @@ template <class Sh, bool COLS, int SIGN> cudaError_t launch_long(const LongPass&
   const size_t smem = Sh::smem_elems() * sizeof(float2);
   const cudaError_t e = allow_smem((const void*)kernel, smem);
   if (e != cudaSuccess) return e;
-  kernel<<<dim3((unsigned)((g.other + Sh::NB - 1) / Sh::NB), B), Sh::NT, smem, st>>>(g);
-  return cudaGetLastError();
+  return launch_next(kernel, dim3((unsigned)((g.other + Sh::NB - 1) / Sh::NB), B), Sh::NT, smem, st, g);
 }
 
 template <class Sh> LongShapeFns rows_only() {

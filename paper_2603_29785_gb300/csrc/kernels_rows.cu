@@ -68,6 +68,7 @@ template <typename V, int E>
 __global__ void k_scale_rows(typename Env<V, E>::S* __restrict__ y, const float* __restrict__ gain, int64_t n_rows,
                              int M) {
   // one block-stride loop per row; rows with gain 1 are left untouched
+  after_previous();
   for (int64_t r = blockIdx.x; r < n_rows; r += gridDim.x) {
     const float g = gain[r];
     if (g == 1.0f) continue;
@@ -102,6 +103,7 @@ template <typename V, int E>
 __global__ void __launch_bounds__(256) k_plane_metrics(const typename Env<V, E>::S* __restrict__ y, int64_t per_plane, int parts,
                                                        double* __restrict__ energy, float* __restrict__ peak) {
   using R = decltype(V().x);
+  after_previous();
   const int64_t pair = blockIdx.x;
   const int64_t len = (per_plane + kMetricParts - 1) / kMetricParts;
   const typename Env<V, E>::S* p = y + pair * per_plane;
@@ -167,6 +169,7 @@ template <typename T> __device__ __forceinline__ int64_t first_largest(const T* 
 __global__ void __launch_bounds__(64) k_best_planes(const double* __restrict__ energy, const float* __restrict__ peak,
                                                     int64_t B, int P, int64_t* __restrict__ best_energy,
                                                     int64_t* __restrict__ best_peak) {
+  after_previous();
   const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
   if (blockIdx.y == 0) best_energy[b] = first_largest(energy + b * P, P);
@@ -178,8 +181,7 @@ __global__ void __launch_bounds__(64) k_best_planes(const double* __restrict__ e
 cudaError_t launch_best_planes(const double* energy, const float* peak, int64_t B, int P, int64_t* best_energy,
                                int64_t* best_peak, cudaStream_t st) {
   if (B == 0) return cudaSuccess;
-  k_best_planes<<<dim3((unsigned)((B + 63) / 64), 2), 64, 0, st>>>(energy, peak, B, P, best_energy, best_peak);
-  return cudaGetLastError();
+  return launch_next(k_best_planes, dim3((unsigned)((B + 63) / 64), 2), 64, 0, st, energy, peak, B, P, best_energy, best_peak);
 }
 
 cudaError_t launch_plane_metrics(const void* y, int env, int64_t pairs, int64_t per_plane, double* energy, float* peak,
@@ -210,16 +212,15 @@ cudaError_t launch_plane_metrics(const void* y, int env, int64_t pairs, int64_t 
 
 cudaError_t launch_scale_rows(void* y, int env, const float* gain, int64_t n_rows, int M, cudaStream_t st) {
   if (n_rows == 0) return cudaSuccess;
-  const unsigned blocks = (unsigned)(n_rows < 65535 ? n_rows : 65535);
+  const dim3 blocks((unsigned)(n_rows < 65535 ? n_rows : 65535));
   switch (env) {
-    case ENV_F64: k_scale_rows<double2, ENV_F64><<<blocks, 256, 0, st>>>(static_cast<double2*>(y), gain, n_rows, M); break;
+    case ENV_F64: return launch_next(k_scale_rows<double2, ENV_F64>, blocks, 256, 0, st, static_cast<double2*>(y), gain, n_rows, M);
     case ENV_BF16:
-      k_scale_rows<float2, ENV_BF16><<<blocks, 256, 0, st>>>(static_cast<__nv_bfloat162*>(y), gain, n_rows, M);
-      break;
-    case ENV_F16: k_scale_rows<float2, ENV_F16><<<blocks, 256, 0, st>>>(static_cast<__half2*>(y), gain, n_rows, M); break;
-    default: k_scale_rows<float2, ENV_F32><<<blocks, 256, 0, st>>>(static_cast<float2*>(y), gain, n_rows, M);
+      return launch_next(k_scale_rows<float2, ENV_BF16>, blocks, 256, 0, st, static_cast<__nv_bfloat162*>(y), gain, n_rows, M);
+    case ENV_F16:
+      return launch_next(k_scale_rows<float2, ENV_F16>, blocks, 256, 0, st, static_cast<__half2*>(y), gain, n_rows, M);
+    default: return launch_next(k_scale_rows<float2, ENV_F32>, blocks, 256, 0, st, static_cast<float2*>(y), gain, n_rows, M);
   }
-  return cudaGetLastError();
 }
 
 // the dense-mode variants follow the ones registered here
@@ -312,9 +313,8 @@ cudaError_t launch_rows_forward(const RowCfg& c, const RowDev<T>* rows, int n_ro
     da.remod = c.remod;
     const cudaError_t e = allow_smem((const void*)k_rows_forward<T, ENV_F64>, c.smem);
     if (e != cudaSuccess) return e;
-    k_rows_forward<T, ENV_F64><<<(unsigned)units, runtime_threads(c, units), c.smem, st>>>(eng, rows, n_rows, Nr, X,
-                                                                           static_cast<double2*>(y), units, twM, wtab, da);
-    return cudaGetLastError();
+    return launch_next(k_rows_forward<T, ENV_F64>, dim3((unsigned)units), runtime_threads(c, units), c.smem, st, eng, rows,
+                       n_rows, Nr, X, static_cast<double2*>(y), units, twM, wtab, da);
   }
 }
 
@@ -348,9 +348,8 @@ cudaError_t launch_rows_inverse(const RowCfg& c, const RowDev<T>* rows, const in
     GenericEngine eng{c.rp};
     const cudaError_t e = allow_smem((const void*)k_rows_inverse<T, ENV_F64>, c.smem);
     if (e != cudaSuccess) return e;
-    k_rows_inverse<T, ENV_F64><<<(unsigned)units, runtime_threads(c, units), c.smem, st>>>(
-        eng, rows, row_list, n_sel, n_rows, Nr, static_cast<const double2*>(y), A, units, twM, wtab, da);
-    return cudaGetLastError();
+    return launch_next(k_rows_inverse<T, ENV_F64>, dim3((unsigned)units), runtime_threads(c, units), c.smem, st, eng, rows,
+                       row_list, n_sel, n_rows, Nr, static_cast<const double2*>(y), A, units, twM, wtab, da);
   }
 }
 

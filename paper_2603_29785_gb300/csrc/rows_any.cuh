@@ -358,7 +358,8 @@ __global__ void __launch_bounds__(Sh::NT, Sh::MINB) k_rows_forward_any(const __g
   if constexpr (NB == 1) {
     int row;
     uint32_t seg;
-    const AnyRow<T> r = any_row<MODE>(g, unit0, Sh::M, false, row, seg);
+    const AnyRow<T> r = any_row<MODE>(g, unit0, Sh::M, false, row, seg);   // tables of the plan
+    after_previous();
     StreamRow<T> s;
     if constexpr (STREAM) s = stream_row(g, row, seg, false);
     any_fft<Sh, +1, T>(
@@ -367,6 +368,7 @@ __global__ void __launch_bounds__(Sh::NT, Sh::MINB) k_rows_forward_any(const __g
   } else {
     __shared__ AnyRow<T> rs[NB];
     __shared__ StreamRow<T> ss[STREAM ? NB : 1];
+    if constexpr (STREAM) after_previous();
     if (threadIdx.x < NB) {
       int row;
       uint32_t seg;
@@ -374,6 +376,7 @@ __global__ void __launch_bounds__(Sh::NT, Sh::MINB) k_rows_forward_any(const __g
       if constexpr (STREAM) ss[threadIdx.x] = stream_row(g, row, seg, false);
     }
     __syncthreads();
+    if constexpr (!STREAM) after_previous();
     any_fft<Sh, +1, T>(
         sm, g.tws, [&](int b, int j, V* a) { load_band<Sh, Sh::R0, T, MODE>(g, rs[b], j, a); },
         [&](int b, int j, V* a) {
@@ -402,6 +405,7 @@ __global__ void __launch_bounds__(Sh::NT, Sh::MINB) k_rows_inverse_any(const __g
     int row;
     uint32_t seg;
     const AnyRow<T> r = any_row<MODE>(g, unit0, Sh::M, true, row, seg);
+    after_previous();
     const int64_t y0 = ((int64_t)seg * g.n_rows + row) * Sh::M;
     StreamRow<T> s;
     if constexpr (STREAM) s = stream_row(g, row, seg, true);
@@ -412,6 +416,7 @@ __global__ void __launch_bounds__(Sh::NT, Sh::MINB) k_rows_inverse_any(const __g
     __shared__ AnyRow<T> rs[NB];
     __shared__ int64_t ys[NB];
     __shared__ StreamRow<T> ss[STREAM ? NB : 1];
+    if constexpr (STREAM) after_previous();
     if (threadIdx.x < NB) {
       int row;
       uint32_t seg;
@@ -420,6 +425,7 @@ __global__ void __launch_bounds__(Sh::NT, Sh::MINB) k_rows_inverse_any(const __g
       if constexpr (STREAM) ss[threadIdx.x] = stream_row(g, row, seg, true);
     }
     __syncthreads();
+    if constexpr (!STREAM) after_previous();
     any_fft<Sh, -1, T>(
         sm, g.tws, [&](int b, int j, V* a) { load(ys[b], rs[b].kc, ss[STREAM ? b : 0], j, a); },
         [&](int b, int j, V* a) { store_band<Sh, RL, T, MODE>(g, rs[b], j, a); });
@@ -432,8 +438,7 @@ cudaError_t launch_any_fwd(const AnyArgs<T>& g, cudaStream_t st) {
   cudaError_t e = allow_smem((const void*)k_rows_forward_any<Sh, T, E, MODE, STREAM>, smem);
   if (e != cudaSuccess) return e;
   const unsigned blocks = (g.n_units + Sh::NB - 1) / Sh::NB;
-  k_rows_forward_any<Sh, T, E, MODE, STREAM><<<blocks, Sh::NT, smem, st>>>(g);
-  return cudaGetLastError();
+  return launch_next(k_rows_forward_any<Sh, T, E, MODE, STREAM>, dim3(blocks), Sh::NT, smem, st, g);
 }
 template <class Sh, typename T, int E, int MODE, bool STREAM = false>
 cudaError_t launch_any_inv(const AnyArgs<T>& g, cudaStream_t st) {
@@ -441,8 +446,7 @@ cudaError_t launch_any_inv(const AnyArgs<T>& g, cudaStream_t st) {
   cudaError_t e = allow_smem((const void*)k_rows_inverse_any<Sh, T, E, MODE, STREAM>, smem);
   if (e != cudaSuccess) return e;
   const unsigned blocks = (g.n_units + Sh::NB - 1) / Sh::NB;
-  k_rows_inverse_any<Sh, T, E, MODE, STREAM><<<blocks, Sh::NT, smem, st>>>(g);
-  return cudaGetLastError();
+  return launch_next(k_rows_inverse_any<Sh, T, E, MODE, STREAM>, dim3(blocks), Sh::NT, smem, st, g);
 }
 
 }  // namespace

@@ -344,6 +344,7 @@ __global__ void __launch_bounds__(kMaxBlock, 1)
     k_rows_forward(GenericEngine eng, const RowDev<T>* __restrict__ rows, int n_rows, int64_t Nr,
                    const cplx<T>* __restrict__ X, typename Env<cplx<T>, E>::S* __restrict__ y, int64_t n_units,
                    const cplx<T>* __restrict__ twM, const T* __restrict__ wtab, DenseArgs<T> da) {
+  after_previous();
   using V = cplx<T>;
   extern __shared__ __align__(16) unsigned char smraw[];
   V* sm = reinterpret_cast<V*>(smraw);
@@ -362,6 +363,7 @@ __global__ void __launch_bounds__(kMaxBlock, 1)
     k_rows_inverse(GenericEngine eng, const RowDev<T>* __restrict__ rows, const int* __restrict__ row_list, int n_sel,
                    int n_rows, int64_t Nr, const typename Env<cplx<T>, E>::S* __restrict__ y, cplx<T>* __restrict__ A,
                    int64_t n_units, const cplx<T>* __restrict__ twM, const T* __restrict__ wtab, DenseArgs<T> da) {
+  after_previous();
   using V = cplx<T>;
   extern __shared__ __align__(16) unsigned char smraw[];
   V* sm = reinterpret_cast<V*>(smraw);
