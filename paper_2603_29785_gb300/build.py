@@ -23,8 +23,10 @@ SOURCES = ["qtam_api.cu", "kernels_long.cu", "kernels_rows.cu", "qtam_noalloc.cu
            "kernels_rows_tuned.cu"]
 PARTS = 16                     # kernels_any.cu compiles once per part (QTAM_PART), in parallel
 LONG_PARTS = 4                 # and kernels_long_any.cu (QTAM_LONG_PART)
+F64_PARTS = 6                  # and kernels_f64.cu (QTAM_F64_PART)
 HEADERS = ["fft_core.cuh", "fft_static.cuh", "qtam_internal.h", "tc_sm100.cuh", "rows_common.cuh", "pair_fft.cuh",
-           "rows_any.cuh", "row_shapes.inc", "kernels_any.cu", "pass_fft.cuh", "long_shapes.inc", "kernels_long_any.cu"]
+           "rows_any.cuh", "row_shapes.inc", "kernels_any.cu", "pass_fft.cuh", "long_shapes.inc", "kernels_long_any.cu",
+           "long_any.cuh", "f64_shapes.inc", "kernels_f64.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
                 "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include")]
@@ -74,6 +76,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     jobs = []
     units = [("kernels_any.cu", f"kernels_any_{k}.o", [f"-DQTAM_PART={k}"]) for k in range(PARTS)]
     units += [("kernels_long_any.cu", f"kernels_long_any_{k}.o", [f"-DQTAM_LONG_PART={k}"]) for k in range(LONG_PARTS)]
+    units += [("kernels_f64.cu", f"kernels_f64_{k}.o", [f"-DQTAM_F64_PART={k}"]) for k in range(F64_PARTS)]
     units += [(s, s.replace(".cu", ".o"), []) for s in SOURCES]
     with cf.ThreadPoolExecutor(max_workers=max(2, os.cpu_count() or 2)) as ex:
         for src, name, defs in units:

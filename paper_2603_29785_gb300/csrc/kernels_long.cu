@@ -292,27 +292,23 @@ void with_engine(const RadixPlan& rp, int nbs, size_t gen_smem, const void* stw,
 // one pass of a batch through its compile-time shape
 template <typename T>
 cudaError_t launch_shape(LongFn f, const LongCfg& c, bool cols, const cplx<T>* in, cplx<T>* out, int64_t nb, cudaStream_t st) {
-  if constexpr (sizeof(T) == 4) {
-    const LongPass g{c.n, cols ? c.n2 : c.n1, in, out, static_cast<const float2*>(c.tw4),
-                     static_cast<const float2*>(cols ? c.stw_col : c.stw_row)};
-    return f(g, (unsigned)nb, st);
-  } else {
-    return cudaErrorNotSupported;
-  }
+  return f(LongPass{c.n, cols ? c.n2 : c.n1, in, out, c.tw4, cols ? c.stw_col : c.stw_row}, (unsigned)nb, st);
 }
 
 }  // namespace
 
-#define QTAM_PARTS(X) X(0) X(1) X(2) X(3)
+#define QTAM_PARTS32(X) X(0) X(1) X(2) X(3)
+#define QTAM_PARTS64(X) X(0) X(1) X(2) X(3) X(4) X(5)
 #define QTAM_DECL(k) const LongShapeFns* long_shapes_##k(int* count);
-QTAM_PARTS(QTAM_DECL)
+QTAM_PARTS32(QTAM_DECL)
 #undef QTAM_DECL
-const LongShapeFns* long_shape(int M) {
-  using Part = const LongShapeFns* (*)(int*);
-#define QTAM_NAME(k) long_shapes_##k,
-  static const Part parts[] = {QTAM_PARTS(QTAM_NAME)};
-#undef QTAM_NAME
-  for (Part part : parts) {
+#define QTAM_DECL(k) const LongShapeFns* f64_long_##k(int* count);
+QTAM_PARTS64(QTAM_DECL)
+#undef QTAM_DECL
+namespace {
+using LongPart = const LongShapeFns* (*)(int*);
+template <size_t N> const LongShapeFns* find_length(const LongPart (&parts)[N], int M) {
+  for (LongPart part : parts) {
     int n = 0;
     const LongShapeFns* s = part(&n);
     for (int i = 0; i < n; ++i)
@@ -320,7 +316,16 @@ const LongShapeFns* long_shape(int M) {
   }
   return nullptr;
 }
-#undef QTAM_PARTS
+}  // namespace
+const LongShapeFns* long_shape(int M, bool f64) {
+#define QTAM_NAME(k) long_shapes_##k,
+  static const LongPart p32[] = {QTAM_PARTS32(QTAM_NAME)};
+#undef QTAM_NAME
+#define QTAM_NAME(k) f64_long_##k,
+  static const LongPart p64[] = {QTAM_PARTS64(QTAM_NAME)};
+#undef QTAM_NAME
+  return f64 ? find_length(p64, M) : find_length(p32, M);
+}
 
 bool long_static_radices(int m, int nbs, int* r, int* nst) {
   if (nbs != kLongColsLog2) return false;

@@ -258,17 +258,37 @@ const AnyShape* any_shape(int M) {
 }
 #undef QTAM_PARTS
 
+#define QTAM_PARTS(X) X(0) X(1) X(2) X(3) X(4) X(5)
+#define QTAM_DECL(k) const F64Rows* f64_rows_##k(int* count);
+QTAM_PARTS(QTAM_DECL)
+#undef QTAM_DECL
+const F64Rows* f64_rows(int M) {
+  using Part = const F64Rows* (*)(int*);
+#define QTAM_NAME(k) f64_rows_##k,
+  static const Part parts[] = {QTAM_PARTS(QTAM_NAME)};
+#undef QTAM_NAME
+  for (Part part : parts) {
+    int n = 0;
+    const F64Rows* s = part(&n);
+    for (int i = 0; i < n; ++i)
+      if (s[i].M == M) return &s[i];
+  }
+  return nullptr;
+}
+#undef QTAM_PARTS
+
 namespace {
 // what forward and inverse launches of the length's own kernels share
-AnyArgs<float> any_args(const RowCfg& c, const RowDev<float>* rows, int n_rows, int n_sel, int64_t Nr, int env, int64_t B,
-                        const float2* twM, const float* wtab) {
-  AnyArgs<float> g{};
+template <typename T>
+AnyArgs<T> any_args(const RowCfg& c, const RowDev<T>* rows, int n_rows, int n_sel, int64_t Nr, int env, int64_t B,
+                    const cplx<T>* twM, const T* wtab) {
+  AnyArgs<T> g{};
   g.rows = rows;
   g.sel = fast_div((uint32_t)n_sel);
   g.n_rows = n_rows;
   g.n_units = (uint32_t)(B * n_sel);
   g.Nr = Nr;
-  g.tws = static_cast<const float2*>(c.any_tw);
+  g.tws = static_cast<const cplx<T>*>(c.any_tw);
   g.wtab = wtab;
   g.twM = twM;
   g.env = env;
@@ -308,6 +328,12 @@ cudaError_t launch_rows_forward(const RowCfg& c, const RowDev<T>* rows, int n_ro
     g.tws = static_cast<const float2*>(c.any_tw_plain);
     return c.any->fwd_plain(g, st);
   } else {
+    if (c.f64) {
+      AnyArgs<T> g = any_args<T>(c, rows, n_rows, n_rows, Nr, env, B, twM, wtab);
+      g.X = X;
+      g.y = y;
+      return c.f64->fwd(g, st);
+    }
     GenericEngine eng{c.rp};
     DenseArgs<T> da;
     da.remod = c.remod;
@@ -345,6 +371,13 @@ cudaError_t launch_rows_inverse(const RowCfg& c, const RowDev<T>* rows, const in
     g.scale = da.scale;
     return plain(g) ? c.any->inv_plain(g, st) : c.any->inv[g.mode](g, st);
   } else {
+    if (c.f64 && !da.divide) {
+      AnyArgs<T> g = any_args<T>(c, rows, n_rows, n_sel, Nr, env, B, twM, wtab);
+      g.row_list = row_list;
+      g.A = A;
+      g.y = const_cast<void*>(y);
+      return c.f64->inv(g, st);
+    }
     GenericEngine eng{c.rp};
     const cudaError_t e = allow_smem((const void*)k_rows_inverse<T, ENV_F64>, c.smem);
     if (e != cudaSuccess) return e;
@@ -357,7 +390,7 @@ cudaError_t launch_rows_stream_forward(const RowCfg& c, const RowDev<float>* row
                                        float2* y, int64_t pitch, int Gm, int Hn, const float2* phase, int64_t B,
                                        cudaStream_t st) {
   if (B * n_rows == 0) return cudaSuccess;
-  AnyArgs<float> g = any_args(c, rows, n_rows, n_rows, Nr, ENV_F32, B, nullptr, nullptr);
+  AnyArgs<float> g = any_args<float>(c, rows, n_rows, n_rows, Nr, ENV_F32, B, nullptr, nullptr);
   g.X = X;
   g.y = y;
   g.pitch = pitch;
@@ -371,7 +404,7 @@ cudaError_t launch_rows_stream_inverse(const RowCfg& c, const RowDev<float>* row
                                        int64_t pitch, int Hn, const float2* phase, float2* A, int64_t B,
                                        cudaStream_t st) {
   if (B * n_sel == 0) return cudaSuccess;
-  AnyArgs<float> g = any_args(c, rows, n_rows, n_sel, Nr, ENV_F32, B, nullptr, nullptr);
+  AnyArgs<float> g = any_args<float>(c, rows, n_rows, n_sel, Nr, ENV_F32, B, nullptr, nullptr);
   g.row_list = row_list;
   g.A = A;
   g.y = const_cast<float2*>(ynew);

@@ -370,25 +370,25 @@ bool choose_long(int64_t n, bool dbl, LongCfg& lc) {
 }
 
 // Build the stage twiddle tables of a compile-time radix sequence in FP64,
-// round to float once and upload them; `pair` writes each entry (c, s) as
+// round to T once and upload them; `pair` writes each entry (c, s) as
 // (c, c, s, s), the layout of the row-pair kernels (one value per row lane).
-qtam_status upload_stage_table(const int* r, int nst, void** dst, size_t& total, bool pair = false) {
+template <typename T> qtam_status upload_stage_table(const int* r, int nst, void** dst, size_t& total, bool pair = false) {
   size_t n = 0;
   stage_twiddles(r, nst, nullptr, &n);
   if (n == 0) n = 1;
   std::vector<double> d(2 * n, 0.0);
   stage_twiddles(r, nst, d.data(), &n);
-  std::vector<float> f;
+  std::vector<T> f;
   if (pair) {
     f.reserve(4 * n);
     for (size_t t = 0; t < n; ++t) {
-      const float c = (float)d[2 * t], s = (float)d[2 * t + 1];
+      const T c = (T)d[2 * t], s = (T)d[2 * t + 1];
       f.insert(f.end(), {c, c, s, s});
     }
   } else {
     f.assign(d.begin(), d.end());
   }
-  return upload(dst, f.data(), f.size() * sizeof(float), total);
+  return upload(dst, f.data(), f.size() * sizeof(T), total);
 }
 
 // round to the nearest BF16, ties to even (finite inputs)
@@ -501,35 +501,40 @@ template <typename T> qtam_status upload_tables(qtam_plan_s* pl) {
   if (pl->rc.tensor && (s = upload_tc_tables(pl, tot)) != QTAM_OK) return s;
   if (sizeof(T) == 4) {
     const AnyShape* sh = pl->rc.any;
-    if ((s = upload_stage_table(sh->r, sh->nst, &pl->d_any_tw, tot)) != QTAM_OK) return s;
-    if ((s = upload_stage_table(sh->r_plain, sh->nst_plain, &pl->d_any_tw_plain, tot)) != QTAM_OK) return s;
+    if ((s = upload_stage_table<T>(sh->r, sh->nst, &pl->d_any_tw, tot)) != QTAM_OK) return s;
+    if ((s = upload_stage_table<T>(sh->r_plain, sh->nst_plain, &pl->d_any_tw_plain, tot)) != QTAM_OK) return s;
     pl->rc.any_tw = pl->d_any_tw;
     pl->rc.any_tw_plain = pl->d_any_tw_plain;
     for (int v = 0; v < row_variant_count(); ++v) {
       const RowVariant* rv = row_variant(v);
       if (rv->M != pl->M) continue;
       void* p = nullptr;
-      if ((s = upload_stage_table(rv->r, rv->nst, &p, tot, rv->tw_pair != 0)) != QTAM_OK) return s;
+      if ((s = upload_stage_table<T>(rv->r, rv->nst, &p, tot, rv->tw_pair != 0)) != QTAM_OK) return s;
       pl->variant_tw[v] = p;
     }
-    // the passes of the long FFT: columns of a power of two have their own engines
-    int r[kMaxStages], nst = 0;
-    const LongShapeFns* ls = long_shape(pl->lc.n1);
-    if (long_static_radices(pl->lc.n1, pl->lc.col_nbs, r, &nst)) {
-      if ((s = upload_stage_table(r, nst, &pl->d_stw_col, tot)) != QTAM_OK) return s;
-    } else if (ls && ls->col_fwd) {
-      if ((s = upload_stage_table(ls->r, ls->nst, &pl->d_stw_col, tot)) != QTAM_OK) return s;
-      pl->lc.cols = ls;
-    }
-    pl->lc.stw_col = pl->d_stw_col;
-    if ((ls = long_shape(pl->lc.n2))) {
-      if ((s = upload_stage_table(ls->r, ls->nst, &pl->d_stw_row, tot)) != QTAM_OK) return s;
-      pl->lc.rows = ls;
-    }
-    pl->lc.stw_row = pl->d_stw_row;
     auto it = pl->variant_tw.find(pl->rc.variant);
     pl->rc.stw = it == pl->variant_tw.end() ? nullptr : it->second;
     if (pl->rc.variant >= 0 && !pl->rc.stw) pl->rc.variant = -1;
+  }
+  {  // the passes of the long FFT: FP32 columns of a power of two have their own engines
+    int r[kMaxStages], nst = 0;
+    const LongShapeFns* ls = long_shape(pl->lc.n1, sizeof(T) == 8);
+    if (sizeof(T) == 4 && long_static_radices(pl->lc.n1, pl->lc.col_nbs, r, &nst)) {
+      if ((s = upload_stage_table<T>(r, nst, &pl->d_stw_col, tot)) != QTAM_OK) return s;
+    } else if (ls && ls->col_fwd) {
+      if ((s = upload_stage_table<T>(ls->r, ls->nst, &pl->d_stw_col, tot)) != QTAM_OK) return s;
+      pl->lc.cols = ls;
+    }
+    pl->lc.stw_col = pl->d_stw_col;
+    if ((ls = long_shape(pl->lc.n2, sizeof(T) == 8))) {
+      if ((s = upload_stage_table<T>(ls->r, ls->nst, &pl->d_stw_row, tot)) != QTAM_OK) return s;
+      pl->lc.rows = ls;
+    }
+    pl->lc.stw_row = pl->d_stw_row;
+  }
+  if (pl->rc.f64) {
+    if ((s = upload_stage_table<T>(pl->rc.f64->r, pl->rc.f64->nst, &pl->d_any_tw, tot)) != QTAM_OK) return s;
+    pl->rc.any_tw = pl->d_any_tw;
   }
   pl->device_bytes += tot;
   return QTAM_OK;
@@ -911,6 +916,7 @@ qtam_status qtam_plan(const qtam_plan_desc* d, int device, qtam_plan_t* out) {
     free_plan(pl);
     return fail(QTAM_ERR_UNSUPPORTED_SIZE, "n_out too large for one thread block");
   }
+  if (dbl && pl->all_bisquare() && pl->eps <= 0 && !pl->remod) pl->rc.f64 = f64_rows(pl->M);
   if (!choose_long(pl->n, dbl, pl->lc)) {
     free_plan(pl);
     return fail(QTAM_ERR_UNSUPPORTED_SIZE, "length/2 must be a product of 2, 3, 5 between 4 and 2^26");

@@ -79,24 +79,25 @@ template <typename T> struct DenseArgs {
 // other = n2 of them) or rows (of length n2, other = n1 of them).
 struct LongPass {
   int n, other;
-  const float2* in;
-  float2* out;
-  const float2* tw4;   // four-step twiddles, [n1][n2]
-  const float2* tws;   // stage twiddles of the length
+  const void* in;    // complex numbers of the kernel's type, all four
+  void* out;
+  const void* tw4;   // four-step twiddles, [n1][n2]
+  const void* tws;   // stage twiddles of the length
 };
 using LongFn = cudaError_t (*)(const LongPass&, unsigned batch, cudaStream_t);
-// Kernels of one sub-length (kernels_long_any.cu, FP32); no column pass above 640.
+// Kernels of one sub-length and type; no column pass above 640.
 struct LongShapeFns {
   int M;
   int nst, r[kMaxStages];
   LongFn col_fwd, col_inv, row_fwd, row_inv;
 };
-// the shape of sub-length M, or nullptr: every 2^a 3^b 5^c from 16 to 1296
-const LongShapeFns* long_shape(int M);
+// the shape of sub-length M in FP32 (kernels_long_any.cu) or FP64 (kernels_f64.cu), or
+// nullptr: every 2^a 3^b 5^c from 16 to 1296
+const LongShapeFns* long_shape(int M, bool f64);
 
 // Long real FFT of N = 2n samples as an n = n1 * n2 four-step complex FFT.
 struct LongCfg {
-  const LongShapeFns* cols = nullptr;   // compile-time passes, where they serve (FP32) ...
+  const LongShapeFns* cols = nullptr;   // compile-time passes, where they serve ...
   const LongShapeFns* rows = nullptr;   // ... else the engines below
   const void* stw_col = nullptr;   // stage twiddle tables of the compile-time column pass (or null)
   const void* stw_row = nullptr;   // ... and row pass
@@ -171,6 +172,16 @@ struct AnyShape {
 // the shape of length M, or nullptr: every 2^a 3^b 5^c from 3 to 7680, and 8192
 const AnyShape* any_shape(int M);
 
+// FP64 rows of bisquare bands (kernels_f64.cu)
+struct F64Rows {
+  int M;
+  int nst, r[kMaxStages];
+  cudaError_t (*fwd)(const AnyArgs<double>&, cudaStream_t);
+  cudaError_t (*inv)(const AnyArgs<double>&, cudaStream_t);
+};
+// those of length M, or nullptr: the lengths of any_shape
+const F64Rows* f64_rows(int M);
+
 struct RowCfg {
   RadixPlan rp;  // radices of M (runtime engine, FP64)
   int threads;
@@ -178,7 +189,8 @@ struct RowCfg {
   int variant;   // index of a registered row-kernel variant, -1 = none
   int chosen = 0;   // launches run that variant (qtam_plan_set_variant), else the length's own shape
   const AnyShape* any = nullptr;   // that shape (FP32 plans) ...
-  const void* any_tw = nullptr;    // ... and its stage twiddles,
+  const F64Rows* f64 = nullptr;    // ... or FP64 rows, where they serve the plan ...
+  const void* any_tw = nullptr;    // ... and the stage twiddles,
   const void* any_tw_plain = nullptr;   // those of the plain forward rows
   int remod = 0; // dense mode: remodulated envelopes
   int floor = 0; // dense mode: stopband floor
