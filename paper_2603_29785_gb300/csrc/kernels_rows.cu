@@ -93,11 +93,20 @@ __global__ void k_scale_rows(typename Env<V, E>::S* __restrict__ y, const float*
 // (non-negative) float bits; both outputs are zeroed by the launcher first.
 //
 // The FP64 pipe (2 lanes a cycle and SM) bounds the reduction, not the read: one
-// block per part spent ten FP64 instructions a warp on two or three elements a
-// thread (128 x 5 planes of 62 x 675: 186 us, 14 % of HBM).  A block now takes
-// `parts` consecutive parts, as many as leave about eight blocks an SM, and
-// reduces once.
+// block per part spent 48 FP64 instructions on two or three elements a thread (128 x 5
+// planes of 62 x 675: 186 us, 14 % of HBM).  A block takes `parts` consecutive parts, as
+// many as leave several waves, and reduces once, in one warp from shared memory (13 FP64
+// instructions, not 48); a partial widens to FP64 in the integer pipe.  scan of those
+// planes 145 -> 137 us, 378 before parts were joined.
 constexpr int kMetricParts = 64;
+
+// (double)x of a sum of squares; normal numbers by moving exponent and fraction
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x);
+  if (u - 0x00800000u >= 0x7f000000u) return (double)x;   // zero, subnormal, infinite, NaN, negative
+  return __hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
 
 template <typename V, int E>
 __global__ void __launch_bounds__(256) k_plane_metrics(const typename Env<V, E>::S* __restrict__ y, int64_t per_plane, int parts,
@@ -123,31 +132,28 @@ __global__ void __launch_bounds__(256) k_plane_metrics(const typename Env<V, E>:
           mx = fmaxf(mx, (float)a2);
         }
       }
-      e += (double)es;
+      e += widen(es);
     }
+  }
+  __shared__ double se[256];
+  __shared__ float sm[256];
+  se[threadIdx.x] = e;
+  sm[threadIdx.x] = mx;
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+#pragma unroll
+  for (int k = 1; k < 8; ++k) {
+    e += se[threadIdx.x + 32 * k];
+    mx = fmaxf(mx, sm[threadIdx.x + 32 * k]);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     e += __shfl_xor_sync(0xffffffffu, e, o);
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   }
-  __shared__ double se[8];
-  __shared__ float sm[8];
-  const int w = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) {
-    se[w] = e;
-    sm[w] = mx;
-  }
-  __syncthreads();
   if (threadIdx.x == 0) {
-    double et = 0.0;
-    float mt = 0.0f;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
-      et += se[k];
-      mt = fmaxf(mt, sm[k]);
-    }
-    atomicAdd(&energy[pair], et);
-    atomicMax(reinterpret_cast<int*>(&peak[pair]), __float_as_int(mt));
+    atomicAdd(&energy[pair], e);
+    atomicMax(reinterpret_cast<int*>(&peak[pair]), __float_as_int(mx));
   }
 }
 
@@ -190,9 +196,10 @@ cudaError_t launch_plane_metrics(const void* y, int env, int64_t pairs, int64_t 
   cudaError_t e0 = cudaMemsetAsync(energy, 0, (size_t)pairs * sizeof(double), st);
   if (e0 == cudaSuccess) e0 = cudaMemsetAsync(peak, 0, (size_t)pairs * sizeof(float), st);
   if (e0 != cudaSuccess) return e0;
-  // a power of two, so that it divides the 64; 1216 = 8 blocks on each of 152 SMs
+  // a power of two, so that it divides the 64; 1216 = 8 blocks on each of 152 SMs, and
+  // at least four such waves, so that a ragged last one costs little
   int parts = 1;
-  while (parts < kMetricParts && pairs * (kMetricParts / parts) >= 2 * 1216) parts *= 2;
+  while (parts < kMetricParts && pairs * (kMetricParts / parts) >= 8 * 1216) parts *= 2;
   const dim3 grid((unsigned)pairs, (unsigned)(kMetricParts / parts));
   switch (env) {
     case ENV_F64:
