@@ -303,6 +303,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     smeta[it][r] = tc_meta_make(ok, seg, row, rows[row], n_rows, Nr, false);
   }
   __syncthreads();
+  after_previous();   // so far only the plan's constants: that overlaps the kernel before
   if (pr < n_pairs) tc_fill_z(sZ, smeta[0], X, wtab);
   tc::fence_smem_to_async();
   tc::fence_before_sync();
@@ -634,6 +635,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     smeta[it][r] = tc_meta_make(ok, seg, row, rows[ok ? row : 0], n_rows, Nr, true);
   }
   __syncthreads();
+  after_previous();
   typename TcLoad<E>::Raw raw[2];
   if (pr < n_pairs) {
 #pragma unroll 1
@@ -792,26 +794,16 @@ cudaError_t launch_rows_forward_tc(const RowCfg& c, const RowDev<float>* rows, i
   const unsigned grid = (unsigned)std::min<int64_t>(pairs, (int64_t)std::max(sms, 1));
   const uint4* A = static_cast<const uint4*>(c.tcA);
   const uint4* G = static_cast<const uint4*>(c.tcG);
-  cudaError_t e;
+  const auto launch = [&](auto kernel, auto* out) {
+    const cudaError_t e = allow_smem((const void*)kernel, kTcSmem);
+    return e == cudaSuccess ? launch_next(kernel, dim3(grid), kTcThreads, kTcSmem, st, rows, n_rows, Nr, X, out, units, A, G, wtab) : e;
+  };
   switch (env) {
-    case ENV_BF16:
-      if ((e = allow_smem((const void*)k_rows_forward_tc<ENV_BF16>, kTcSmem)) != cudaSuccess) return e;
-      k_rows_forward_tc<ENV_BF16><<<grid, kTcThreads, kTcSmem, st>>>(
-          rows, n_rows, Nr, X, static_cast<__nv_bfloat162*>(y), units, A, G, wtab);
-      break;
-    case ENV_F16:
-      if ((e = allow_smem((const void*)k_rows_forward_tc<ENV_F16>, kTcSmem)) != cudaSuccess) return e;
-      k_rows_forward_tc<ENV_F16><<<grid, kTcThreads, kTcSmem, st>>>(rows, n_rows, Nr, X, static_cast<__half2*>(y),
-                                                                    units, A, G, wtab);
-      break;
-    default:
-      if ((e = allow_smem((const void*)k_rows_forward_tc<ENV_F32>, kTcSmem)) != cudaSuccess) return e;
-      k_rows_forward_tc<ENV_F32><<<grid, kTcThreads, kTcSmem, st>>>(rows, n_rows, Nr, X, static_cast<float2*>(y),
-                                                                    units, A, G, wtab);
+    case ENV_BF16: return launch(k_rows_forward_tc<ENV_BF16>, static_cast<__nv_bfloat162*>(y));
+    case ENV_F16: return launch(k_rows_forward_tc<ENV_F16>, static_cast<__half2*>(y));
+    default: return launch(k_rows_forward_tc<ENV_F32>, static_cast<float2*>(y));
   }
-  return cudaGetLastError();
 }
-
 
 bool launch_rows_inverse_tc(const RowCfg& c, const RowDev<float>* rows, const int* row_list, int n_sel, int n_rows,
                             int64_t Nr, const void* y, int env, float2* A, int64_t B, cudaStream_t st,
@@ -827,27 +819,17 @@ bool launch_rows_inverse_tc(const RowCfg& c, const RowDev<float>* rows, const in
   const unsigned grid = (unsigned)std::min<int64_t>(pairs, (int64_t)std::max(sms, 1));
   const uint4* Ai = static_cast<const uint4*>(c.tcAi);
   const uint4* G = static_cast<const uint4*>(c.tcG);
-  cudaError_t e;
+  const auto launch = [&](auto kernel, const auto* in) {
+    const cudaError_t e = allow_smem((const void*)kernel, kTcSmem);
+    return e == cudaSuccess ? launch_next(kernel, dim3(grid), kTcThreads, kTcSmem, st, rows, row_list, n_sel, n_rows, Nr, in, A, units,
+                                          Ai, G, wtab)
+                            : e;
+  };
   switch (env) {
-    case ENV_BF16:
-      if ((e = allow_smem((const void*)k_rows_inverse_tc<ENV_BF16>, kTcSmem)) != cudaSuccess) break;
-      k_rows_inverse_tc<ENV_BF16><<<grid, kTcThreads, kTcSmem, st>>>(
-          rows, row_list, n_sel, n_rows, Nr, static_cast<const __nv_bfloat162*>(y), A, units, Ai, G, wtab);
-      e = cudaGetLastError();
-      break;
-    case ENV_F16:
-      if ((e = allow_smem((const void*)k_rows_inverse_tc<ENV_F16>, kTcSmem)) != cudaSuccess) break;
-      k_rows_inverse_tc<ENV_F16><<<grid, kTcThreads, kTcSmem, st>>>(
-          rows, row_list, n_sel, n_rows, Nr, static_cast<const __half2*>(y), A, units, Ai, G, wtab);
-      e = cudaGetLastError();
-      break;
-    default:
-      if ((e = allow_smem((const void*)k_rows_inverse_tc<ENV_F32>, kTcSmem)) != cudaSuccess) break;
-      k_rows_inverse_tc<ENV_F32><<<grid, kTcThreads, kTcSmem, st>>>(
-          rows, row_list, n_sel, n_rows, Nr, static_cast<const float2*>(y), A, units, Ai, G, wtab);
-      e = cudaGetLastError();
+    case ENV_BF16: *err = launch(k_rows_inverse_tc<ENV_BF16>, static_cast<const __nv_bfloat162*>(y)); break;
+    case ENV_F16: *err = launch(k_rows_inverse_tc<ENV_F16>, static_cast<const __half2*>(y)); break;
+    default: *err = launch(k_rows_inverse_tc<ENV_F32>, static_cast<const float2*>(y));
   }
-  *err = e;
   return true;
 }
 
