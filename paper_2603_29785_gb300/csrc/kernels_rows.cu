@@ -82,6 +82,21 @@ __global__ void k_scale_rows(typename Env<V, E>::S* __restrict__ y, const float*
   }
 }
 
+// Zeroes 8-byte words.  A kernel, not a memset node, so that it is set up while the
+// kernel before drains and the accumulation while it drains; 16-byte stores between an
+// odd first and last word.  Pair of one 64 s segment 47 -> 43.5 us, uneven graph 276 -> 270.
+__global__ void __launch_bounds__(256) k_zero(uint2* __restrict__ p, int64_t words) {
+  after_previous();
+  const int64_t head = (reinterpret_cast<uintptr_t>(p) & 8) && words > 0 ? 1 : 0, quads = (words - head) / 2;
+  uint4* q = reinterpret_cast<uint4*>(p + head);
+  const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x, stride = (int64_t)gridDim.x * 256;
+  if (t == 0) {
+    if (head) p[0] = make_uint2(0u, 0u);
+    if (head + 2 * quads < words) p[words - 1] = make_uint2(0u, 0u);
+  }
+  for (int64_t i = t; i < quads; i += stride) q[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 // Per (segment, plane) pair: energy = sum |Y|^2 and peak = max |Y|^2 over
 // the K*M envelope values (App. A optimal-plane selection).  FP32 envelopes are
 // squared in FP32 and summed in FP32 partials of at most 8 terms (relative
@@ -157,6 +172,15 @@ __global__ void __launch_bounds__(256) k_plane_metrics(const typename Env<V, E>:
   }
 }
 
+__global__ void __launch_bounds__(256) k_clear_metrics(double* __restrict__ energy, float* __restrict__ peak, int64_t pairs) {
+  after_previous();
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (i < pairs) {
+    energy[i] = 0.0;
+    peak[i] = 0.0f;
+  }
+}
+
 // One thread per segment and metric over the segment's few planes: both choices in
 // one launch of the latency of a single load chain (2 us; two general arg-max
 // reductions took 7.4 + 3.5 us for 128 x 5 planes).
@@ -184,6 +208,12 @@ __global__ void __launch_bounds__(64) k_best_planes(const double* __restrict__ e
 
 }  // namespace
 
+cudaError_t launch_zero(void* p, size_t bytes, cudaStream_t st) {
+  if (bytes == 0) return cudaSuccess;
+  const int64_t words = (int64_t)(bytes / 8), blocks = (words + 2047) / 2048;   // four 16-byte stores a thread
+  return launch_next(k_zero, dim3((unsigned)(blocks < 152 * 64 ? blocks : 152 * 64)), 256, 0, st, static_cast<uint2*>(p), words);
+}
+
 cudaError_t launch_best_planes(const double* energy, const float* peak, int64_t B, int P, int64_t* best_energy,
                                int64_t* best_peak, cudaStream_t st) {
   if (B == 0) return cudaSuccess;
@@ -193,28 +223,22 @@ cudaError_t launch_best_planes(const double* energy, const float* peak, int64_t 
 cudaError_t launch_plane_metrics(const void* y, int env, int64_t pairs, int64_t per_plane, double* energy, float* peak,
                                  cudaStream_t st) {
   if (pairs == 0) return cudaSuccess;
-  cudaError_t e0 = cudaMemsetAsync(energy, 0, (size_t)pairs * sizeof(double), st);
-  if (e0 == cudaSuccess) e0 = cudaMemsetAsync(peak, 0, (size_t)pairs * sizeof(float), st);
+  const cudaError_t e0 = launch_next(k_clear_metrics, dim3((unsigned)((pairs + 255) / 256)), 256, 0, st, energy, peak, pairs);
   if (e0 != cudaSuccess) return e0;
   // a power of two, so that it divides the 64; 1216 = 8 blocks on each of 152 SMs, and
   // at least four such waves, so that a ragged last one costs little
   int parts = 1;
   while (parts < kMetricParts && pairs * (kMetricParts / parts) >= 8 * 1216) parts *= 2;
   const dim3 grid((unsigned)pairs, (unsigned)(kMetricParts / parts));
+  const auto launch = [&](auto kernel, const auto* p) {
+    return launch_next(kernel, grid, 256, 0, st, p, per_plane, parts, energy, peak);
+  };
   switch (env) {
-    case ENV_F64:
-      k_plane_metrics<double2, ENV_F64><<<grid, 256, 0, st>>>(static_cast<const double2*>(y), per_plane, parts, energy, peak);
-      break;
-    case ENV_BF16:
-      k_plane_metrics<float2, ENV_BF16><<<grid, 256, 0, st>>>(static_cast<const __nv_bfloat162*>(y), per_plane, parts, energy, peak);
-      break;
-    case ENV_F16:
-      k_plane_metrics<float2, ENV_F16><<<grid, 256, 0, st>>>(static_cast<const __half2*>(y), per_plane, parts, energy, peak);
-      break;
-    default:
-      k_plane_metrics<float2, ENV_F32><<<grid, 256, 0, st>>>(static_cast<const float2*>(y), per_plane, parts, energy, peak);
+    case ENV_F64: return launch(k_plane_metrics<double2, ENV_F64>, static_cast<const double2*>(y));
+    case ENV_BF16: return launch(k_plane_metrics<float2, ENV_BF16>, static_cast<const __nv_bfloat162*>(y));
+    case ENV_F16: return launch(k_plane_metrics<float2, ENV_F16>, static_cast<const __half2*>(y));
+    default: return launch(k_plane_metrics<float2, ENV_F32>, static_cast<const float2*>(y));
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_scale_rows(void* y, int env, const float* gain, int64_t n_rows, int M, cudaStream_t st) {

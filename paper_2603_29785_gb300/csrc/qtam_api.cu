@@ -644,8 +644,8 @@ template <typename T> qtam_status run_envelopes(qtam_plan_s* pl, const void* X, 
 template <typename T>
 qtam_status run_accumulate(qtam_plan_s* pl, const void* y, int64_t B, const MaskEntry* me, void* A, cudaStream_t st) {
   using V = cplx<T>;
-  cudaError_t e = cudaMemsetAsync(A, 0, (size_t)B * pl->Nr * sizeof(V), st);
-  if (e != cudaSuccess) return fail_cuda(e, "cudaMemsetAsync");
+  cudaError_t e = launch_zero(A, (size_t)B * pl->Nr * sizeof(V), st);
+  if (e != cudaSuccess) return fail_cuda(e, "clearing the accumulator");
   if constexpr (sizeof(T) == 4) {
     if (pl->rc.tensor &&
         launch_rows_inverse_tc(pl->rc, static_cast<const RowDev<float>*>(pl->d_rows), me->rows, me->n_sel,
@@ -717,7 +717,7 @@ qtam_status stream_inverse_fused(qtam_plan_s* pl, const void* hist, int hcols, c
   if (s != QTAM_OK) return s;
   DeviceGuard g(pl->device);
   Regions rg = split_ws(pl, ws, b);
-  cudaError_t e = cudaMemsetAsync(rg.r0, 0, (size_t)b * pl->Nr * sizeof(float2), st);
+  cudaError_t e = launch_zero(rg.r0, (size_t)b * pl->Nr * sizeof(float2), st);
   if (e == cudaSuccess)
     e = launch_rows_stream_inverse(pl->rc, static_cast<const RowDev<float>*>(pl->d_rows), me->rows, me->n_sel,
                                    pl->P * pl->K, pl->Nr, static_cast<const float2*>(hist), hcols,

@@ -275,6 +275,8 @@ qtam_status stream_inverse_fused(qtam_plan_s* pl, const void* hist, int hcols, c
                                  cudaStream_t st, bool* used);
 
 int row_variant_count();
+// `bytes` (a multiple of 8) zeroes at p, aligned to 8
+cudaError_t launch_zero(void* p, size_t bytes, cudaStream_t st);
 // per (segment, plane) pair: energy = sum |Y|^2 (FP64), peak = max |Y|^2 over K*M values
 cudaError_t launch_plane_metrics(const void* y, int env, int64_t pairs, int64_t per_plane, double* energy, float* peak,
                                  cudaStream_t st);
