@@ -72,8 +72,8 @@ template <typename V> struct StoreRowsTransposed {
 };
 
 template <class Eng, typename T>
-__global__ void __launch_bounds__(Eng::NT, Eng::MINB) k_col_forward(Eng eng, int n, int n2, const cplx<T>* __restrict__ z,
-                                                          cplx<T>* __restrict__ U, const cplx<T>* __restrict__ tw4,
+__global__ void __launch_bounds__(Eng::NT, Eng::MINB) k_col_forward(Eng eng, int n, int n2, const cplx<T>* z,
+                                                          cplx<T>* U, const cplx<T>* __restrict__ tw4,
                                                           const cplx<T>* __restrict__ ftw) {
   using V = cplx<T>;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -87,8 +87,8 @@ __global__ void __launch_bounds__(Eng::NT, Eng::MINB) k_col_forward(Eng eng, int
 }
 
 template <class Eng, typename T>
-__global__ void __launch_bounds__(Eng::NT, Eng::MINB) k_row_forward(Eng eng, int n, int n1, const cplx<T>* __restrict__ U,
-                                                          cplx<T>* __restrict__ Z, const cplx<T>* __restrict__ ftw) {
+__global__ void __launch_bounds__(Eng::NT, Eng::MINB) k_row_forward(Eng eng, int n, int n1, const cplx<T>* U,
+                                                          cplx<T>* Z, const cplx<T>* __restrict__ ftw) {
   using V = cplx<T>;
   extern __shared__ __align__(16) unsigned char smraw[];
   V* sm = reinterpret_cast<V*>(smraw);
@@ -108,38 +108,45 @@ template <typename V> __device__ __forceinline__ V wN(const V* twN, int n, int k
 }
 
 // (k, n-k) pairs a thread and threads a block.  FP32: four, for memory-level
-// parallelism.  FP64: one, in small blocks, because the FP64 pipe (2 lanes a cycle and
-// SM) bounds it and 1024 pairs a block left all but five SMs idle at n = 8192 (8.4 us).
+// parallelism: all loaded before the first is stored, for the kernel may not claim that
+// its input and its output never alias (launch_next).  FP64: one, in small blocks,
+// because the FP64 pipe (2 lanes a cycle and SM) bounds it and 1024 pairs a block left
+// all but five SMs idle at n = 8192 (8.4 us).
 template <typename T> struct Untangle {
   static constexpr int PAIRS = sizeof(T) == 8 ? 1 : 4, NT = sizeof(T) == 8 ? 64 : 256;
   static dim3 grid(int n, int64_t nb) { return dim3((unsigned)((n / 2 + 1 + NT * PAIRS - 1) / (NT * PAIRS)), (unsigned)nb); }
 };
 
 template <typename T>
-__global__ void k_untangle_forward(int n, const cplx<T>* __restrict__ Z, cplx<T>* __restrict__ X,
-                                   const cplx<T>* __restrict__ twN) {
+__global__ void k_untangle_forward(int n, const cplx<T>* Z, cplx<T>* X, const cplx<T>* __restrict__ twN) {
   using V = cplx<T>;
   after_previous();
   const int64_t seg = blockIdx.y;
   const V* Zs = Z + seg * n;
   V* Xs = X + seg * (int64_t)(n + 1);
   const T half = (T)0.5;
-  const int base = blockIdx.x * blockDim.x * Untangle<T>::PAIRS + threadIdx.x;
+  constexpr int PAIRS = Untangle<T>::PAIRS;
+  const int base = blockIdx.x * blockDim.x * PAIRS + threadIdx.x;
+  V zk[PAIRS], zm[PAIRS];
 #pragma unroll
-  for (int u = 0; u < Untangle<T>::PAIRS; ++u) {
-    const int k = base + u * blockDim.x;
+  for (int u = 0; u < PAIRS; ++u) {
+    const int k = base + u * blockDim.x, kk = n - k;   // partner bin, in [n/2, n]
     if (k > (n >> 1)) break;
-    const int kk = n - k;                     // partner bin, in [n/2, n]
-    const V zk = Zs[k];
-    const V zm = Zs[kk == n ? 0 : kk];
+    zk[u] = Zs[k];
+    zm[u] = Zs[kk == n ? 0 : kk];
+  }
+#pragma unroll
+  for (int u = 0; u < PAIRS; ++u) {
+    const int k = base + u * blockDim.x, kk = n - k;
+    if (k > (n >> 1)) break;
     {
-      const V a = zk, b = cconj(zm);
+      const V a = zk[u], b = cconj(zm[u]);
       const V s = a + b, d = a - b;
       const V t = cmul(__ldg(&twN[k]), d);    // w^k (a - b)
       Xs[k] = mk<V>(half * (s.x + t.y), half * (s.y - t.x));   // s/2 - (i/2) t
     }
     if (kk != k) {
-      const V a = zm, b = cconj(zk);
+      const V a = zm[u], b = cconj(zk[u]);
       const V s = a + b, d = a - b;
       const V t = cmul(wN(twN, n, kk), d);
       Xs[kk] = mk<V>(half * (s.x + t.y), half * (s.y - t.x));
@@ -161,22 +168,30 @@ __device__ __forceinline__ cplx<T> zi_value(cplx<T> xk, cplx<T> xm, cplx<T> wk, 
 }
 
 template <typename T>
-__global__ void k_untangle_inverse(int n, const cplx<T>* __restrict__ A, const T* __restrict__ invP,
-                                   cplx<T>* __restrict__ Zi, const cplx<T>* __restrict__ twN, T scale) {
+__global__ void k_untangle_inverse(int n, const cplx<T>* A, const T* __restrict__ invP, cplx<T>* Zi,
+                                   const cplx<T>* __restrict__ twN, T scale) {
   using V = cplx<T>;
   after_previous();
   const int64_t seg = blockIdx.y;
   const V* As = A + seg * (int64_t)(n + 1);
   V* Zs = Zi + seg * n;
   const T hs = (T)0.5 * scale;
-  const int base = blockIdx.x * blockDim.x * Untangle<T>::PAIRS + threadIdx.x;
+  constexpr int PAIRS = Untangle<T>::PAIRS;
+  const int base = blockIdx.x * blockDim.x * PAIRS + threadIdx.x;
+  V ak[PAIRS], am[PAIRS];
 #pragma unroll
-  for (int u = 0; u < Untangle<T>::PAIRS; ++u) {
-    const int k = base + u * blockDim.x;
+  for (int u = 0; u < PAIRS; ++u) {
+    const int k = base + u * blockDim.x, kk = n - k;   // kk in [n/2, n]
     if (k > (n >> 1)) break;
-    const int kk = n - k;                     // in [n/2, n]
-    V xk = cscale(As[k], __ldg(&invP[k]));
-    V xm = cscale(As[kk], __ldg(&invP[kk]));
+    ak[u] = As[k];
+    am[u] = As[kk];
+  }
+#pragma unroll
+  for (int u = 0; u < PAIRS; ++u) {
+    const int k = base + u * blockDim.x, kk = n - k;
+    if (k > (n >> 1)) break;
+    V xk = cscale(ak[u], __ldg(&invP[k]));
+    V xm = cscale(am[u], __ldg(&invP[kk]));
     if (k == 0) xk.y = (T)0;
     if (kk == n) xm.y = (T)0;
     const V wk = __ldg(&twN[k]);
@@ -203,8 +218,8 @@ template <typename V> struct StoreColumns {
 };
 
 template <class Eng, typename T>
-__global__ void __launch_bounds__(Eng::NT, Eng::MINB) k_row_inverse(Eng eng, int n, int n1, const cplx<T>* __restrict__ Zi,
-                                                          cplx<T>* __restrict__ Vb, const cplx<T>* __restrict__ tw4,
+__global__ void __launch_bounds__(Eng::NT, Eng::MINB) k_row_inverse(Eng eng, int n, int n1, const cplx<T>* Zi,
+                                                          cplx<T>* Vb, const cplx<T>* __restrict__ tw4,
                                                           const cplx<T>* __restrict__ ftw) {
   using V = cplx<T>;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -218,8 +233,8 @@ __global__ void __launch_bounds__(Eng::NT, Eng::MINB) k_row_inverse(Eng eng, int
 }
 
 template <class Eng, typename T>
-__global__ void __launch_bounds__(Eng::NT, Eng::MINB) k_col_inverse(Eng eng, int n, int n2, const cplx<T>* __restrict__ Vb,
-                                                          cplx<T>* __restrict__ xout, const cplx<T>* __restrict__ ftw) {
+__global__ void __launch_bounds__(Eng::NT, Eng::MINB) k_col_inverse(Eng eng, int n, int n2, const cplx<T>* Vb,
+                                                          cplx<T>* xout, const cplx<T>* __restrict__ ftw) {
   using V = cplx<T>;
   extern __shared__ __align__(16) unsigned char smraw[];
   V* sm = reinterpret_cast<V*>(smraw);

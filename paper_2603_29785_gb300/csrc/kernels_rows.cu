@@ -65,8 +65,7 @@ const RowVariant kVariants[] = {
 #undef QTAM_VT
 
 template <typename V, int E>
-__global__ void k_scale_rows(typename Env<V, E>::S* __restrict__ y, const float* __restrict__ gain, int64_t n_rows,
-                             int M) {
+__global__ void k_scale_rows(typename Env<V, E>::S* y, const float* gain, int64_t n_rows, int M) {
   // one block-stride loop per row; rows with gain 1 are left untouched
   after_previous();
   for (int64_t r = blockIdx.x; r < n_rows; r += gridDim.x) {
@@ -85,7 +84,7 @@ __global__ void k_scale_rows(typename Env<V, E>::S* __restrict__ y, const float*
 // Zeroes 8-byte words.  A kernel, not a memset node, so that it is set up while the
 // kernel before drains and the accumulation while it drains; 16-byte stores between an
 // odd first and last word.  Pair of one 64 s segment 47 -> 43.5 us, uneven graph 276 -> 270.
-__global__ void __launch_bounds__(256) k_zero(uint2* __restrict__ p, int64_t words) {
+__global__ void __launch_bounds__(256) k_zero(uint2* p, int64_t words) {
   after_previous();
   const int64_t head = (reinterpret_cast<uintptr_t>(p) & 8) && words > 0 ? 1 : 0, quads = (words - head) / 2;
   uint4* q = reinterpret_cast<uint4*>(p + head);
@@ -124,8 +123,8 @@ __device__ __forceinline__ double widen(float x) {
 __device__ __forceinline__ double widen(double x) { return x; }
 
 template <typename V, int E>
-__global__ void __launch_bounds__(256) k_plane_metrics(const typename Env<V, E>::S* __restrict__ y, int64_t per_plane, int parts,
-                                                       double* __restrict__ energy, float* __restrict__ peak) {
+__global__ void __launch_bounds__(256) k_plane_metrics(const typename Env<V, E>::S* y, int64_t per_plane, int parts, double* energy,
+                                                       float* peak) {
   using R = decltype(V().x);
   after_previous();
   const int64_t pair = blockIdx.x;
@@ -172,7 +171,7 @@ __global__ void __launch_bounds__(256) k_plane_metrics(const typename Env<V, E>:
   }
 }
 
-__global__ void __launch_bounds__(256) k_clear_metrics(double* __restrict__ energy, float* __restrict__ peak, int64_t pairs) {
+__global__ void __launch_bounds__(256) k_clear_metrics(double* energy, float* peak, int64_t pairs) {
   after_previous();
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (i < pairs) {
@@ -184,7 +183,7 @@ __global__ void __launch_bounds__(256) k_clear_metrics(double* __restrict__ ener
 // One thread per segment and metric over the segment's few planes: both choices in
 // one launch of the latency of a single load chain (2 us; two general arg-max
 // reductions took 7.4 + 3.5 us for 128 x 5 planes).
-template <typename T> __device__ __forceinline__ int64_t first_largest(const T* __restrict__ v, int n) {
+template <typename T> __device__ __forceinline__ int64_t first_largest(const T* v, int n) {
   int best = 0;
   T m = v[0];
   for (int i = 1; i < n; ++i) {
@@ -196,9 +195,8 @@ template <typename T> __device__ __forceinline__ int64_t first_largest(const T* 
   }
   return best;
 }
-__global__ void __launch_bounds__(64) k_best_planes(const double* __restrict__ energy, const float* __restrict__ peak,
-                                                    int64_t B, int P, int64_t* __restrict__ best_energy,
-                                                    int64_t* __restrict__ best_peak) {
+__global__ void __launch_bounds__(64) k_best_planes(const double* energy, const float* peak, int64_t B, int P,
+                                                    int64_t* best_energy, int64_t* best_peak) {
   after_previous();
   const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;

@@ -186,7 +186,7 @@ __device__ __forceinline__ bool tc_meta_unit_fwd(int64_t pk, int r, int64_t n_pa
 // ((tid >> 7) & 1, tid & 127, tid >> 8) loads Z[r][128 j1 + j2] for j1 in
 // 32 h .. 32 h + 31: a warp's loads are 32 consecutive bins, its 16-byte
 // stores one core-matrix row each.
-__device__ __forceinline__ void tc_fill_z(unsigned char* sZ, const TcMeta* meta, const float2* __restrict__ X,
+__device__ __forceinline__ void tc_fill_z(unsigned char* sZ, const TcMeta* meta, const float2* X,
                                           const float* __restrict__ wtab) {
   const int tid = threadIdx.x;
   const int r = (tid >> 7) & 1, j2 = tid & 127, h0 = 4 * (tid >> 8);
@@ -239,7 +239,7 @@ __device__ __forceinline__ void tc_fill_z(unsigned char* sZ, const TcMeta* meta,
 // burst of stores from every SM at once.
 template <int E>
 __device__ __forceinline__ void tc_store_y(uint32_t tbase, int64_t pr, int64_t n_units,
-                                           typename TcEnv<E>::S* __restrict__ y, int q0, int q1) {
+                                           typename TcEnv<E>::S* y, int q0, int q1) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q4 = warp & 3, quarter = warp >> 2;   // lane quarter, quarter of the n2 range
   const int r = q4 >> 1, n1 = 32 * (q4 & 1) + lane;
@@ -261,8 +261,8 @@ __device__ __forceinline__ void tc_store_y(uint32_t tbase, int64_t pr, int64_t n
 
 template <int E>
 __global__ void __launch_bounds__(kTcThreads, 1)
-    k_rows_forward_tc(const RowDev<float>* __restrict__ rows, int n_rows, int64_t Nr, const float2* __restrict__ X,
-                      typename TcEnv<E>::S* __restrict__ y, int64_t n_units, const uint4* __restrict__ tabA,
+    k_rows_forward_tc(const RowDev<float>* __restrict__ rows, int n_rows, int64_t Nr, const float2* X,
+                      typename TcEnv<E>::S* y, int64_t n_units, const uint4* __restrict__ tabA,
                       const uint4* __restrict__ tabG, const float* __restrict__ wtab) {
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ __align__(8) uint64_t mbarA, mbarB;
@@ -554,7 +554,7 @@ __device__ __forceinline__ void tc_store_row(unsigned char* sY, int r, bool vali
 // Warp (q4, quarter) reads lanes j2 = 32 q4 + lane of row r = quarter >> 1,
 // j1 in 32 (quarter & 1) .. + 31; blocks of 16 j1 wholly outside the band
 // are skipped by the whole warp.
-__device__ __forceinline__ void tc_accumulate(uint32_t tbase, const TcMeta* meta, float2* __restrict__ A,
+__device__ __forceinline__ void tc_accumulate(uint32_t tbase, const TcMeta* meta, float2* A,
                                               const float* __restrict__ wtab) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q4 = warp & 3, quarter = warp >> 2;
@@ -594,7 +594,7 @@ __device__ __forceinline__ void tc_accumulate(uint32_t tbase, const TcMeta* meta
 template <int E>
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_rows_inverse_tc(const RowDev<float>* __restrict__ rows, const int* __restrict__ row_list, int n_sel, int n_rows,
-                      int64_t Nr, const typename TcEnv<E>::S* __restrict__ y, float2* __restrict__ A, int64_t n_units,
+                      int64_t Nr, const typename TcEnv<E>::S* y, float2* A, int64_t n_units,
                       const uint4* __restrict__ tabAi, const uint4* __restrict__ tabG, const float* __restrict__ wtab) {
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ __align__(8) uint64_t mbarA, mbarB;

@@ -24,7 +24,9 @@ inline cudaError_t allow_smem(const void* fn, size_t bytes) {
 
 // Launch that may be set up while the kernel before it in the stream drains; every
 // thread of the kernel calls after_previous() before it touches anything an earlier
-// kernel wrote or reads.  A call is four or five dependent kernels, and each gap of
+// kernel wrote or reads, and takes such buffers without __restrict__: earlier kernels
+// write them while it runs, and the promise would let the compiler read them through the
+// non-coherent path or ahead of the wait.  Tables uploaded before the launch may carry it.  A call is four or five dependent kernels, and each gap of
 // about 1.5 us closes: pair of one 64 s segment 58 -> 47 us, of 16 with five windows
 // 325 -> 304, forward of 64 535 -> 522, uneven graph 291 -> 276.
 template <class... P, class... A>

@@ -82,8 +82,8 @@ __device__ __forceinline__ void carrier_phase(int64_t kc, int64_t a, int64_t N, 
 // chunks of 262144 samples 4.9 us, 14.9 with one flat index and single samples.
 constexpr int kGatherPer = 4;
 template <typename V>
-__global__ void __launch_bounds__(256) k_stream_gather_x(const V* __restrict__ hist, int64_t nh, const V* __restrict__ xnew,
-                                                         int64_t hop, int64_t N, V* __restrict__ chunks) {
+__global__ void __launch_bounds__(256) k_stream_gather_x(const V* hist, int64_t nh, const V* xnew, int64_t hop, int64_t N,
+                                                         V* chunks) {
   qtam::after_previous();
   const int64_t i = blockIdx.y, t0 = (int64_t)blockIdx.x * (256 * kGatherPer) + threadIdx.x;
   V v[kGatherPer];
@@ -158,7 +158,7 @@ __global__ void k_stream_gather_y(const S* __restrict__ hist, int hcols, const S
 // took 5.6 us on 40 SMs).
 constexpr int kPhaseThreads = 32;
 __global__ void __launch_bounds__(kPhaseThreads) k_stream_phases(const int* __restrict__ kc, int R, int64_t b, int64_t N, int64_t a0, int64_t hop,
-                                double sign, float2* __restrict__ phase) {
+                                double sign, float2* phase) {
   qtam::after_previous();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= b * R) return;

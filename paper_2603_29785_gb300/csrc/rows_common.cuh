@@ -342,7 +342,7 @@ __device__ __forceinline__ void rows_inverse_body(const Eng& eng, const RowDev<T
 template <typename T, int E>
 __global__ void __launch_bounds__(kMaxBlock, 1)
     k_rows_forward(GenericEngine eng, const RowDev<T>* __restrict__ rows, int n_rows, int64_t Nr,
-                   const cplx<T>* __restrict__ X, typename Env<cplx<T>, E>::S* __restrict__ y, int64_t n_units,
+                   const cplx<T>* X, typename Env<cplx<T>, E>::S* y, int64_t n_units,
                    const cplx<T>* __restrict__ twM, const T* __restrict__ wtab, DenseArgs<T> da) {
   after_previous();
   using V = cplx<T>;
@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(kMaxBlock, 1)
 template <typename T, int E>
 __global__ void __launch_bounds__(kMaxBlock, 1)
     k_rows_inverse(GenericEngine eng, const RowDev<T>* __restrict__ rows, const int* __restrict__ row_list, int n_sel,
-                   int n_rows, int64_t Nr, const typename Env<cplx<T>, E>::S* __restrict__ y, cplx<T>* __restrict__ A,
+                   int n_rows, int64_t Nr, const typename Env<cplx<T>, E>::S* y, cplx<T>* A,
                    int64_t n_units, const cplx<T>* __restrict__ twM, const T* __restrict__ wtab, DenseArgs<T> da) {
   after_previous();
   using V = cplx<T>;
