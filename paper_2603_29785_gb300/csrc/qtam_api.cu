@@ -268,6 +268,14 @@ qtam_status upload(void** dst, const void* src, size_t bytes, size_t& total) {
   if (e != cudaSuccess) return fail_cuda(e, "cudaMemcpy");
   return QTAM_OK;
 }
+// Waits for the copies of upload().  Their source is pageable, so cudaMemcpy may return
+// while the device still copies out of the driver's staging buffer, and a launch on a
+// non-blocking stream does not wait for the legacy stream: the row kernels read their
+// tables even before the kernel ahead of them has finished.
+qtam_status finish_uploads() {
+  const cudaError_t e = cudaStreamSynchronize(cudaStreamLegacy);
+  return e == cudaSuccess ? QTAM_OK : fail_cuda(e, "uploading tables");
+}
 
 // Build (or find) the normaliser and row list for a plane mask.  Called with plan->mu held.
 qtam_status build_mask(qtam_plan_s* pl, uint64_t mask, MaskEntry** out) {
@@ -317,10 +325,11 @@ qtam_status build_mask(qtam_plan_s* pl, uint64_t mask, MaskEntry** out) {
       std::vector<float> invf(inv.begin(), inv.end());
       s = upload(&e.invP, invf.data(), invf.size() * sizeof(float), tot);
     }
-    if (s != QTAM_OK) return s;
-    s = upload(reinterpret_cast<void**>(&e.rows), rows.data(), rows.size() * sizeof(int), tot);
+    if (s == QTAM_OK) s = upload(reinterpret_cast<void**>(&e.rows), rows.data(), rows.size() * sizeof(int), tot);
+    if (s == QTAM_OK) s = finish_uploads();
     if (s != QTAM_OK) {
       cudaFree(e.invP);
+      cudaFree(e.rows);
       return s;
     }
     pl->device_bytes += tot;
@@ -537,7 +546,7 @@ template <typename T> qtam_status upload_tables(qtam_plan_s* pl) {
     pl->rc.any_tw = pl->d_any_tw;
   }
   pl->device_bytes += tot;
-  return QTAM_OK;
+  return finish_uploads();
 }
 
 // A compile-time row variant serves a plan of its length with FP32 compute;

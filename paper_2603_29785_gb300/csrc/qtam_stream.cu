@@ -371,6 +371,9 @@ qtam_status qtam_stream_create(qtam_plan_t plan, int64_t hop, int64_t max_chunks
     if (hxb) e = cudaMemset(s->hx[i], 0, hxb);
     if (e == cudaSuccess && hyb) e = cudaMemset(s->hy[i], 0, hyb);
   }
+  // the copy's source is pageable and a memset returns at once: neither is ordered with
+  // the launches of a non-blocking stream
+  if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
   if (e != cudaSuccess) {
     free_stream(s);
     return sfail_cuda(e, "stream setup");

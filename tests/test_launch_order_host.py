@@ -3,7 +3,10 @@
 Until such a kernel has passed after_previous(), earlier kernels write the buffers
 it works on.  A ``__restrict__`` pointer promises the compiler that nobody else does:
 it may then read through the non-coherent path, or move an access over the wait.  Only
-tables that are complete before any launch (the plan's and the mask's) may carry it."""
+tables that are complete before any launch (the plan's and the mask's) may carry it, and
+what uploads them waits for its copies: cudaMemcpy from pageable memory and cudaMemset
+may return before the device has them, and non-blocking streams do not wait for the
+legacy stream."""
 import glob
 import os
 import re
@@ -85,3 +88,19 @@ def test_only_tables_are_restrict(kernel):
             assert promised <= TABLES, (kernel, file, name, sorted(promised - TABLES))
             # and what it calls, by name
             todo += [w for w in set(re.findall(r"\b(\w+)\s*(?:<[^;(){}]*>)?\(", body)) if w in by_name and w not in seen]
+
+
+@pytest.mark.parametrize("file,function,wait", [("qtam_api.cu", "upload_tables", "return finish_uploads();"),
+                                                ("qtam_api.cu", "build_mask", "s = finish_uploads();"),
+                                                ("qtam_stream.cu", "qtam_stream_create",
+                                                 "e = cudaStreamSynchronize(cudaStreamLegacy);")])
+def test_uploads_are_complete_before_the_handle_is_out(file, function, wait):
+    text = open(os.path.join(build.CSRC, file)).read()
+    m = re.search(r"\bqtam_status\s+" + function + r"\(", text)
+    body = text[m.start():_closing(text, text.index("{", m.start()), "{}")]
+    copies = [c.start() for c in re.finditer(r"\bupload\w*(?:<\w+>)?\(|cudaMem(?:cpy|set)\(", body)]
+    waits = [w.start() for w in re.finditer(re.escape(wait), body)]
+    assert waits and max(copies[1:] or copies) < max(waits)
+    if "finish" in wait:
+        f = re.search(r"qtam_status finish_uploads\(\) \{(.*?)\n\}", text, re.S)
+        assert "cudaStreamSynchronize(cudaStreamLegacy)" in f.group(1)
