@@ -463,7 +463,7 @@ class Plan:
         r = qtam_plan_rows(self.handle, self.P * self.K)
         shp = (self.P, self.K)
         self.geometry = Geometry(r["f"].reshape(shp), r["kc"].reshape(shp), r["h"].reshape(shp), r["c"].reshape(shp))
-        self._ws = {}
+        self._ws = threading.local()   # .by_stream: this thread's scratch, {stream handle: tensor}
         self._need = (-1, 0)     # workspace bytes of the last batch size asked for
 
     def __del__(self):
@@ -476,17 +476,40 @@ class Plan:
     def frame_operator(self, plane_mask: int = 0) -> np.ndarray:
         return qtam_frame_operator(self.handle, plane_mask, self.Nr)
 
-    def workspace(self, batch: int):
-        import torch
+    def workspace(self, batch: int, stream=None):
+        """(scratch tensor, its bytes) for `batch` segments on `stream` (default: the current one).
+
+        Calls that may run at the same time need scratch of their own, so a plan keeps one buffer for
+        each stream a thread uses (at most MAX_SCRATCH a thread, the oldest given back first): work on
+        one stream is ordered, and two threads may interleave the kernels of their calls on one.  A
+        buffer is allocated on its stream, so that dropping it is ordered with the kernels using it."""
         last, need = self._need
         if last != batch:
             need = qtam_workspace_size(self.handle, batch)
             self._need = (batch, need)
-        ws = self._ws.get(self.device)
+        st = _stream(stream) or 0
+        try:
+            mine = self._ws.by_stream
+        except AttributeError:
+            mine = self._ws.by_stream = {}
+        ws = mine.get(st)
         if ws is None or ws.numel() < need:
-            ws = torch.empty(max(need, 256), dtype=torch.uint8, device=f"cuda:{self.device}")
-            self._ws[self.device] = ws
+            mine.pop(st, None)
+            while len(mine) >= self.MAX_SCRATCH:
+                del mine[next(iter(mine))]
+            ws = mine[st] = self._scratch(max(need, 256), st)
         return ws, ws.numel()
+
+    MAX_SCRATCH = 32     # as many streams as PyTorch's pool hands out
+
+    def _scratch(self, nbytes, st):
+        import torch
+        dev = torch.device("cuda", self.device)
+        if torch.cuda.current_stream(dev).cuda_stream == st:
+            return torch.empty(nbytes, dtype=torch.uint8, device=dev)
+        own = torch.cuda.ExternalStream(st, device=dev) if st else torch.cuda.default_stream(dev)
+        with torch.cuda.stream(own):
+            return torch.empty(nbytes, dtype=torch.uint8, device=dev)
 
     def real_dtype(self):
         import torch
@@ -533,7 +556,8 @@ class Plan:
         y = self.envelope_tensor(B) if y is None else self._check_y(y)
         if y.shape[0] != B:
             raise ValueError("x and y batch sizes differ")
-        ws, wsb = self.workspace(B)
+        stream = _stream(stream)
+        ws, wsb = self.workspace(B, stream)
         qtam_forward(self.handle, x, B, y, ws, wsb, stream)
         return y
 
@@ -544,7 +568,8 @@ class Plan:
         x = torch.empty((B, self.N), dtype=self.real_dtype(), device=y.device) if x is None else self._check_x(x)
         if x.shape[0] != B:
             raise ValueError("x and y batch sizes differ")
-        ws, wsb = self.workspace(B)
+        stream = _stream(stream)
+        ws, wsb = self.workspace(B, stream)
         qtam_inverse(self.handle, y, B, plane_mask, x, ws, wsb, stream)
         return x
 
@@ -554,7 +579,8 @@ class Plan:
         self._check_y(y)
         B = y.shape[0]
         x = torch.empty((B, self.N), dtype=self.real_dtype(), device=y.device) if x is None else self._check_x(x)
-        ws, wsb = self.workspace(B)
+        stream = _stream(stream)
+        ws, wsb = self.workspace(B, stream)
         qtam_inverse_single_tile(self.handle, y, B, plane, row, x, ws, wsb, stream)
         return x
 
@@ -586,7 +612,8 @@ class Plan:
         B = x.shape[0]
         cdt = torch.complex128 if self.compute == "f64" else torch.complex64
         X = torch.empty((B, self.Nr), dtype=cdt, device=x.device)
-        ws, wsb = self.workspace(B)
+        stream = _stream(stream)
+        ws, wsb = self.workspace(B, stream)
         qtam_stage_spectrum(self.handle, x, B, X, ws, wsb, stream)
         return X
 
@@ -610,7 +637,8 @@ class Plan:
         self._check_spec(A, "A")
         B = A.shape[0]
         x = torch.empty((B, self.N), dtype=self.real_dtype(), device=A.device)
-        ws, wsb = self.workspace(B)
+        stream = _stream(stream)
+        ws, wsb = self.workspace(B, stream)
         qtam_stage_synthesize(self.handle, A, B, plane_mask, x, ws, wsb, stream)
         return x
 
