@@ -425,6 +425,26 @@ def _require(t, shape, dtypes, device, name):
         raise ValueError(f"{name} must be a contiguous cuda:{device} tensor {want} of {dtypes}; got {got}")
 
 
+def _empty(shape, dtype, device, stream=None):
+    """An uninitialised tensor on cuda:`device` for kernels on `stream` (None: the current one).
+
+    For another stream it is allocated there: the current stream's free blocks may still be in use by
+    kernels queued on it.  It is also recorded on the current stream, where the caller will read it, so that
+    dropping it waits for both."""
+    import torch
+    if stream is None:
+        return torch.empty(shape, dtype=dtype, device=f"cuda:{device}")
+    dev = torch.device("cuda", device)
+    st = _stream(stream) or 0
+    cur = torch.cuda.current_stream(dev)
+    if cur.cuda_stream == st:
+        return torch.empty(shape, dtype=dtype, device=dev)
+    with torch.cuda.stream(torch.cuda.ExternalStream(st, device=dev) if st else torch.cuda.default_stream(dev)):
+        t = torch.empty(shape, dtype=dtype, device=dev)
+    t.record_stream(cur)
+    return t
+
+
 # ----------------------------------------------------------------------------
 # convenience wrapper
 # ----------------------------------------------------------------------------
@@ -504,27 +524,21 @@ class Plan:
 
     def _scratch(self, nbytes, st):
         import torch
-        dev = torch.device("cuda", self.device)
-        if torch.cuda.current_stream(dev).cuda_stream == st:
-            return torch.empty(nbytes, dtype=torch.uint8, device=dev)
-        own = torch.cuda.ExternalStream(st, device=dev) if st else torch.cuda.default_stream(dev)
-        with torch.cuda.stream(own):
-            return torch.empty(nbytes, dtype=torch.uint8, device=dev)
+        return _empty(nbytes, torch.uint8, self.device, st)
 
     def real_dtype(self):
         import torch
         return torch.float64 if self.compute == "f64" else torch.float32
 
-    def envelope_tensor(self, batch: int):
+    def envelope_tensor(self, batch: int, stream=None):
         import torch
-        dev = f"cuda:{self.device}"
         shp = (batch, self.P, self.K, self.M)
         if self.envelope == "f32":
-            return torch.empty(shp, dtype=torch.complex64, device=dev)
+            return _empty(shp, torch.complex64, self.device, stream)
         if self.envelope == "f64":
-            return torch.empty(shp, dtype=torch.complex128, device=dev)
+            return _empty(shp, torch.complex128, self.device, stream)
         dt = torch.bfloat16 if self.envelope == "bf16" else torch.float16
-        return torch.empty(shp + (2,), dtype=dt, device=dev)
+        return _empty(shp + (2,), dt, self.device, stream)
 
     def _check_x(self, x):
         if x.dim() == 1:
@@ -553,7 +567,7 @@ class Plan:
     def forward(self, x, y=None, stream=None):
         x = self._check_x(x)
         B = x.shape[0]
-        y = self.envelope_tensor(B) if y is None else self._check_y(y)
+        y = self.envelope_tensor(B, stream) if y is None else self._check_y(y)
         if y.shape[0] != B:
             raise ValueError("x and y batch sizes differ")
         stream = _stream(stream)
@@ -562,10 +576,9 @@ class Plan:
         return y
 
     def inverse(self, y, plane_mask: int = 0, x=None, stream=None):
-        import torch
         self._check_y(y)
         B = y.shape[0]
-        x = torch.empty((B, self.N), dtype=self.real_dtype(), device=y.device) if x is None else self._check_x(x)
+        x = _empty((B, self.N), self.real_dtype(), self.device, stream) if x is None else self._check_x(x)
         if x.shape[0] != B:
             raise ValueError("x and y batch sizes differ")
         stream = _stream(stream)
@@ -575,10 +588,9 @@ class Plan:
 
     def inverse_single_tile(self, y, plane: int, row: int, x=None, stream=None):
         """Dense mode: reconstruct every segment from its one tile (plane, row)."""
-        import torch
         self._check_y(y)
         B = y.shape[0]
-        x = torch.empty((B, self.N), dtype=self.real_dtype(), device=y.device) if x is None else self._check_x(x)
+        x = _empty((B, self.N), self.real_dtype(), self.device, stream) if x is None else self._check_x(x)
         stream = _stream(stream)
         ws, wsb = self.workspace(B, stream)
         qtam_inverse_single_tile(self.handle, y, B, plane, row, x, ws, wsb, stream)
@@ -590,10 +602,10 @@ class Plan:
         import torch
         self._check_y(y)
         B = y.shape[0]
-        energy = torch.empty((B, self.P), dtype=torch.float64, device=y.device)
-        peak = torch.empty((B, self.P), dtype=torch.float32, device=y.device)
-        best_energy = torch.empty((B,), dtype=torch.int64, device=y.device)
-        best_peak = torch.empty((B,), dtype=torch.int64, device=y.device)
+        energy = _empty((B, self.P), torch.float64, self.device, stream)
+        peak = _empty((B, self.P), torch.float32, self.device, stream)
+        best_energy = _empty((B,), torch.int64, self.device, stream)
+        best_peak = _empty((B,), torch.int64, self.device, stream)
         qtam_plane_metrics(self.handle, y, B, energy, peak, stream)
         qtam_best_planes(self.handle, energy, peak, B, best_energy, best_peak, stream)
         return energy, peak, best_energy, best_peak
@@ -607,11 +619,9 @@ class Plan:
         return y
 
     def spectrum(self, x, stream=None):
-        import torch
         x = self._check_x(x)
         B = x.shape[0]
-        cdt = torch.complex128 if self.compute == "f64" else torch.complex64
-        X = torch.empty((B, self.Nr), dtype=cdt, device=x.device)
+        X = _empty((B, self.Nr), self.complex_dtype(), self.device, stream)
         stream = _stream(stream)
         ws, wsb = self.workspace(B, stream)
         qtam_stage_spectrum(self.handle, x, B, X, ws, wsb, stream)
@@ -620,23 +630,21 @@ class Plan:
     def envelopes(self, X, stream=None):
         self._check_spec(X, "X")
         B = X.shape[0]
-        y = self.envelope_tensor(B)
+        y = self.envelope_tensor(B, stream)
         qtam_stage_envelopes(self.handle, X, B, y, stream)
         return y
 
     def accumulate(self, y, plane_mask: int = 0, stream=None):
-        import torch
         self._check_y(y)
         B = y.shape[0]
-        A = torch.empty((B, self.Nr), dtype=self.complex_dtype(), device=y.device)
+        A = _empty((B, self.Nr), self.complex_dtype(), self.device, stream)
         qtam_stage_accumulate(self.handle, y, B, plane_mask, A, stream)
         return A
 
     def synthesize(self, A, plane_mask: int = 0, stream=None):
-        import torch
         self._check_spec(A, "A")
         B = A.shape[0]
-        x = torch.empty((B, self.N), dtype=self.real_dtype(), device=A.device)
+        x = _empty((B, self.N), self.real_dtype(), self.device, stream)
         stream = _stream(stream)
         ws, wsb = self.workspace(B, stream)
         qtam_stage_synthesize(self.handle, A, B, plane_mask, x, ws, wsb, stream)
@@ -667,17 +675,16 @@ class Stream:
         except Exception:
             pass
 
-    def _map_tensor(self, cols):
+    def _map_tensor(self, cols, stream=None):
         import torch
         p = self.plan
-        dev = f"cuda:{p.device}"
         shp = (p.P, p.K, cols)
         if p.envelope == "f32":
-            return torch.empty(shp, dtype=torch.complex64, device=dev)
+            return _empty(shp, torch.complex64, p.device, stream)
         if p.envelope == "f64":
-            return torch.empty(shp, dtype=torch.complex128, device=dev)
+            return _empty(shp, torch.complex128, p.device, stream)
         dt = torch.bfloat16 if p.envelope == "bf16" else torch.float16
-        return torch.empty(shp + (2,), dtype=dt, device=dev)
+        return _empty(shp + (2,), dt, p.device, stream)
 
     def forward(self, x, stream=None):
         p = self.plan
@@ -685,7 +692,7 @@ class Stream:
         n = int(x.shape[0])
         if n % self.hop:
             raise ValueError(f"push a multiple of hop = {self.hop} samples; got {n}")
-        y = self._map_tensor(n // self.hop * self.hop_cols)
+        y = self._map_tensor(n // self.hop * self.hop_cols, stream)
         qtam_stream_forward(self.handle, x, n, y, stream)
         return y
 
@@ -700,7 +707,7 @@ class Stream:
         cols = int(y.shape[2])
         if cols % self.hop_cols:
             raise ValueError(f"push a multiple of {self.hop_cols} map columns; got {cols}")
-        x = torch.empty((cols // self.hop_cols * self.hop,), dtype=p.real_dtype(), device=y.device)
+        x = _empty((cols // self.hop_cols * self.hop,), p.real_dtype(), p.device, stream)
         qtam_stream_inverse(self.handle, y, cols, plane_mask, x, stream)
         return x
 

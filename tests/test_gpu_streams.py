@@ -87,3 +87,32 @@ def test_new_tables_on_a_non_blocking_stream(compute):
         assert torch.equal(y, wy) and same(xh, wx, tol)
         st0 = qtam.Stream(old, max_chunks=2)
         assert torch.equal(z, st0.forward(x[0, :st0.hop].clone()))
+
+
+def test_outputs_belong_to_the_stream_that_writes_them():
+    """A block freed on the current stream, whose kernels may not have run, is not handed to a call on
+    another stream; an output read on the current stream is not reused by its own before that has run."""
+    p = qtam.Plan(*ARGS, device=0)
+    x = inputs(p, 1)[0]
+    s = torch.cuda.Stream()
+    want = p.forward(x)
+    p.forward(x, stream=s)
+    torch.cuda.synchronize()
+    old = p.envelope_tensor(6)
+    at = old.data_ptr()
+    del old
+    y = p.forward(x, stream=s)
+    assert y.data_ptr() != at
+    del y
+    outs = [p.forward(x, stream=s), p.inverse(want, stream=s), p.spectrum(x, stream=s), *p.plane_metrics(want, stream=s)]
+    s.synchronize()
+    assert torch.equal(outs[0], want) and same(outs[1], p.inverse(want)) and torch.equal(outs[2], p.spectrum(x))
+    assert all(torch.equal(a, b) for a, b in zip(outs[4:], p.plane_metrics(want)[1:]))
+    at = outs[0].data_ptr()
+    torch.cuda._sleep(20_000_000)                    # the current stream is busy about 10 ms
+    twice = outs[0] + outs[0]
+    del outs
+    y = p.forward(x, stream=s)
+    assert y.data_ptr() != at
+    torch.cuda.synchronize()
+    assert torch.equal(twice, want + want)
