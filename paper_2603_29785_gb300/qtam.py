@@ -591,6 +591,8 @@ class Plan:
         self._check_y(y)
         B = y.shape[0]
         x = _empty((B, self.N), self.real_dtype(), self.device, stream) if x is None else self._check_x(x)
+        if x.shape[0] != B:
+            raise ValueError("x and y batch sizes differ")
         stream = _stream(stream)
         ws, wsb = self.workspace(B, stream)
         qtam_inverse_single_tile(self.handle, y, B, plane, row, x, ws, wsb, stream)

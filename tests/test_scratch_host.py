@@ -44,3 +44,38 @@ def test_growth_and_bound(plan):
         plan.workspace(1, s)
     assert plan.workspace(1, 100)[0] is first and plan.workspace(1, 5)[0] is not b     # the oldest went first
     assert len(plan._ws.by_stream) == plan.MAX_SCRATCH
+
+
+class FakeTensor:
+    """What the argument checks read of a device tensor (of a host-only plan's device, -1)."""
+    is_cuda = True
+
+    def __init__(self, shape, dtype):
+        self.shape, self.dtype = shape, dtype
+
+    def get_device(self):
+        return -1
+
+    def is_contiguous(self):
+        return True
+
+    def dim(self):
+        return len(self.shape)
+
+    def data_ptr(self):
+        return 256
+
+
+def test_single_tile_output_holds_the_batch(monkeypatch):
+    """The kernels write B segments: an output with fewer is refused before they are launched."""
+    torch = pytest.importorskip("torch")
+    monkeypatch.setattr(qtam.Plan, "_scratch", lambda self, nbytes, st: FakeTensor((nbytes,), torch.uint8), raising=False)
+    monkeypatch.setattr(FakeTensor, "numel", lambda self: self.shape[0], raising=False)
+    monkeypatch.setattr(qtam, "_stream", lambda s: s or 0)
+    p = qtam.Plan(64.0, 256, (3.0,), 2.0, 31.0, 5, n_out=135, stopband_eps=1e-3, device=-1)
+    y = FakeTensor((3, p.P, p.K, p.M), torch.complex64)
+    with pytest.raises(ValueError, match="batch sizes differ"):
+        p.inverse_single_tile(y, 0, 1, x=FakeTensor((2, p.N), torch.float32))
+    with pytest.raises(qtam.QtamError) as e:           # the right size reaches the library, which has no device
+        p.inverse_single_tile(y, 0, 1, x=FakeTensor((3, p.N), torch.float32))
+    assert e.value.status == 8
