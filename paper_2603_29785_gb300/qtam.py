@@ -484,7 +484,7 @@ class Plan:
         shp = (self.P, self.K)
         self.geometry = Geometry(r["f"].reshape(shp), r["kc"].reshape(shp), r["h"].reshape(shp), r["c"].reshape(shp))
         self._ws = threading.local()   # .by_stream: this thread's scratch, {stream handle: tensor}
-        self._need = (-1, 0)     # workspace bytes of the last batch size asked for
+        self._need = (None, 0)   # workspace bytes of the last batch size asked for
 
     def __del__(self):
         try:

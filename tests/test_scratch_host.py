@@ -79,3 +79,10 @@ def test_single_tile_output_holds_the_batch(monkeypatch):
     with pytest.raises(qtam.QtamError) as e:           # the right size reaches the library, which has no device
         p.inverse_single_tile(y, 0, 1, x=FakeTensor((3, p.N), torch.float32))
     assert e.value.status == 8
+
+
+def test_negative_batch_is_refused(plan):
+    for _ in range(2):
+        with pytest.raises(qtam.QtamError) as e:
+            plan.workspace(-1, 11)
+        assert e.value.status == 1
