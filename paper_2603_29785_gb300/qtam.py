@@ -159,17 +159,12 @@ def _ptr(t) -> int | None:
     raise TypeError(f"cannot pass {type(t)} as a pointer")
 
 
-try:
-    from torch._C import _cuda_getCurrentRawStream as _raw_stream
-except ImportError:        # host-only PyTorch, or none
-    _raw_stream = None
-
-
 def _stream(stream) -> int | None:
     if stream is None:
         import torch
-        if _raw_stream is not None and torch.cuda.is_initialized():
-            return _raw_stream(torch.cuda.current_device())    # without a Stream object per call
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)     # absent from host-only PyTorch
+        if raw is not None and torch.cuda.is_initialized():
+            return raw(torch.cuda.current_device())    # without a Stream object per call
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream

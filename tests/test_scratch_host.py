@@ -86,3 +86,12 @@ def test_negative_batch_is_refused(plan):
         with pytest.raises(qtam.QtamError) as e:
             plan.workspace(-1, 11)
         assert e.value.status == 1
+
+
+def test_the_binding_loads_without_pytorch():
+    """Geometry and planning on the host need no device memory, so no import of PyTorch (seconds)."""
+    import subprocess
+    import sys
+    code = ("import sys; from paper_2603_29785_gb300 import qtam; p = qtam.Plan(4096.0, 16384, (8.0,), 20.0, 1024.0, 16, "
+            "device=-1); p.frame_operator(); assert 'torch' not in sys.modules")
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=qtam._build.ROOT)
