@@ -275,24 +275,23 @@ int gen_nbs(int nbs, int64_t count, int64_t batch) {
   return nbs;
 }
 
-#define QTAM_CASE(M, ...)                                       \
-  case M: {                                                     \
-    using E = StatLong<M, __VA_ARGS__>;                         \
-    f(E(), E::smem_bytes(sizeof(float2)), (const cplx<T>*)stw); \
-    return;                                                     \
+#define QTAM_CASE(M, ...)                                              \
+  case M: {                                                            \
+    using E = StatLong<M, __VA_ARGS__>;                                \
+    return f(E(), E::smem_bytes(sizeof(float2)), (const cplx<T>*)stw); \
   }
 
-// Call f(engine, smem bytes, engine twiddles): the static column engine where the
+// The result of f(engine, smem bytes, engine twiddles): the static column engine where the
 // plan built its tables (stw), else the runtime engine with the length-n table.
 template <typename T, class F>
-void with_engine(const RadixPlan& rp, int nbs, size_t gen_smem, const void* stw, const cplx<T>* twn, int count, int64_t batch,
+cudaError_t with_engine(const RadixPlan& rp, int nbs, size_t gen_smem, const void* stw, const cplx<T>* twn, int count, int64_t batch,
                  F&& f) {
   if constexpr (sizeof(T) == 4) {
     if (stw) {
       switch (rp.m) { QTAM_LONG_CASES(QTAM_CASE) default: break; }
     }
   }
-  f(GenLong{rp, gen_nbs(nbs, count, batch)}, gen_smem, twn);
+  return f(GenLong{rp, gen_nbs(nbs, count, batch)}, gen_smem, twn);
 }
 #undef QTAM_CASE
 
@@ -360,27 +359,31 @@ cudaError_t launch_spectrum(const LongCfg& c, const cplx<T>* z, cplx<T>* U, cplx
       const cudaError_t e = launch_shape<T>(c.cols->col_fwd, c, true, z + off, U + off, nb, st);
       if (e != cudaSuccess) return e;
     } else {
-      with_engine<T>(c.rp1, c.col_nbs, c.col_smem, c.stw_col, twn, c.n2, nb, [&](auto eng, size_t smem, const cplx<T>* ftw) {
+      const cudaError_t e = with_engine<T>(c.rp1, c.col_nbs, c.col_smem, c.stw_col, twn, c.n2, nb,
+                                              [&](auto eng, size_t smem, const cplx<T>* ftw) {
         using E = decltype(eng);
         dim3 g(c.n2 >> eng.nb_shift(), (unsigned)nb);
-        launch_pass(k_col_forward<E, T>, eng, smem, g, st, c.n, c.n2, z + off, U + off, tw4, ftw);
+        return launch_pass(k_col_forward<E, T>, eng, smem, g, st, c.n, c.n2, z + off, U + off, tw4, ftw);
       });
+      if (e != cudaSuccess) return e;
     }
     if (c.rows) {
       const cudaError_t e = launch_shape<T>(c.rows->row_fwd, c, false, (const cplx<T>*)(U + off), Z + off, nb, st);
       if (e != cudaSuccess) return e;
     } else {
-      with_engine<T>(c.rp2, c.row_nbs, c.row_smem, nullptr, twn, c.n1, nb, [&](auto eng, size_t smem, const cplx<T>* ftw) {
+      const cudaError_t e = with_engine<T>(c.rp2, c.row_nbs, c.row_smem, nullptr, twn, c.n1, nb,
+                                              [&](auto eng, size_t smem, const cplx<T>* ftw) {
         using E = decltype(eng);
         dim3 g(c.n1 >> eng.nb_shift(), (unsigned)nb);
-        launch_pass(k_row_forward<E, T>, eng, smem, g, st, c.n, c.n1, (const cplx<T>*)(U + off), Z + off, ftw);
+        return launch_pass(k_row_forward<E, T>, eng, smem, g, st, c.n, c.n1, (const cplx<T>*)(U + off), Z + off, ftw);
       });
+      if (e != cudaSuccess) return e;
     }
     const cudaError_t e = launch_next(k_untangle_forward<T>, Untangle<T>::grid(c.n, nb), Untangle<T>::NT, 0, st, c.n, Z + off,
                                       X + s0 * (int64_t)(c.n + 1), twN);
     if (e != cudaSuccess) return e;
   }
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 template <typename T>
@@ -397,24 +400,28 @@ cudaError_t launch_synthesis(const LongCfg& c, const cplx<T>* A, const T* invP, 
       const cudaError_t e = launch_shape<T>(c.rows->row_inv, c, false, (const cplx<T>*)(Zi + off), Vb + off, nb, st);
       if (e != cudaSuccess) return e;
     } else {
-      with_engine<T>(c.rp2, c.row_nbs, c.row_smem, nullptr, twn, c.n1, nb, [&](auto eng, size_t smem, const cplx<T>* ftw) {
+      const cudaError_t e = with_engine<T>(c.rp2, c.row_nbs, c.row_smem, nullptr, twn, c.n1, nb,
+                                              [&](auto eng, size_t smem, const cplx<T>* ftw) {
         using E = decltype(eng);
         dim3 g(c.n1 >> eng.nb_shift(), (unsigned)nb);
-        launch_pass(k_row_inverse<E, T>, eng, smem, g, st, c.n, c.n1, (const cplx<T>*)(Zi + off), Vb + off, tw4, ftw);
+        return launch_pass(k_row_inverse<E, T>, eng, smem, g, st, c.n, c.n1, (const cplx<T>*)(Zi + off), Vb + off, tw4, ftw);
       });
+      if (e != cudaSuccess) return e;
     }
     if (c.cols) {
       const cudaError_t e = launch_shape<T>(c.cols->col_inv, c, true, (const cplx<T>*)(Vb + off), xout + off, nb, st);
       if (e != cudaSuccess) return e;
     } else {
-      with_engine<T>(c.rp1, c.col_nbs, c.col_smem, c.stw_col, twn, c.n2, nb, [&](auto eng, size_t smem, const cplx<T>* ftw) {
+      const cudaError_t e = with_engine<T>(c.rp1, c.col_nbs, c.col_smem, c.stw_col, twn, c.n2, nb,
+                                              [&](auto eng, size_t smem, const cplx<T>* ftw) {
         using E = decltype(eng);
         dim3 g(c.n2 >> eng.nb_shift(), (unsigned)nb);
-        launch_pass(k_col_inverse<E, T>, eng, smem, g, st, c.n, c.n2, (const cplx<T>*)(Vb + off), xout + off, ftw);
+        return launch_pass(k_col_inverse<E, T>, eng, smem, g, st, c.n, c.n2, (const cplx<T>*)(Vb + off), xout + off, ftw);
       });
+      if (e != cudaSuccess) return e;
     }
   }
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 template cudaError_t launch_spectrum<float>(const LongCfg&, const float2*, float2*, float2*, float2*, int64_t,

@@ -38,13 +38,15 @@ namespace {
 
 thread_local std::string g_last_error;
 
+// A CUDA error is reported once: the runtime keeps it until it is read, and the next
+// launch that asks cudaGetLastError() would report it again.
 qtam_status fail(qtam_status s, const std::string& msg) {
   g_last_error = msg;
+  if (s == QTAM_ERR_CUDA || s == QTAM_ERR_OUT_OF_MEMORY) (void)cudaGetLastError();
   return s;
 }
 qtam_status fail_cuda(cudaError_t e, const char* where) {
-  g_last_error = std::string(where) + ": " + cudaGetErrorString(e);
-  return QTAM_ERR_CUDA;
+  return fail(QTAM_ERR_CUDA, std::string(where) + ": " + cudaGetErrorString(e));
 }
 
 constexpr int kMaxSmem = 227 * 1024;

@@ -191,11 +191,11 @@ cudaError_t gather_y(const void* hist, int hcols, const void* ynew, int64_t pitc
 
 qtam_status sfail(qtam_status s, const std::string& msg) {
   qtam::set_last_error(msg);
+  if (s == QTAM_ERR_CUDA || s == QTAM_ERR_OUT_OF_MEMORY) (void)cudaGetLastError();   // reported once
   return s;
 }
 qtam_status sfail_cuda(cudaError_t e, const char* where) {
-  qtam::set_last_error(std::string(where) + ": " + cudaGetErrorString(e));
-  return QTAM_ERR_CUDA;
+  return sfail(QTAM_ERR_CUDA, std::string(where) + ": " + cudaGetErrorString(e));
 }
 
 struct DevScope {
