@@ -162,9 +162,9 @@ typedef struct {
   double kappa;                   /* max over kept bins of max_k W_k / P (all planes) */
   int64_t kept_bins;              /* |F_tau| for all planes */
   int64_t device_bytes;           /* bytes of resident plan tables on the device */
-  int32_t row_variant;            /* registered CUDA-core row variant of the plan's length (its first choice
-                                     before tuning), -1 if none; launches run the length's own
-                                     kernels until qtam_plan_set_variant chooses a variant */
+  int32_t row_variant;            /* first registered CUDA-core row variant of the plan's length, -1 if none,
+                                     and the chosen one after qtam_plan_set_variant; what launches run
+                                     is qtam_plan_running_variant */
   int32_t short_dft;              /* QTAM_SHORT_DFT_* engine of the envelope stage */
   double stopband_eps;            /* dense mode floor (0: off) */
   int32_t remodulate;             /* 1: envelopes carry the carrier exp(+2 pi i k_c n / M) */
@@ -201,9 +201,17 @@ QTAM_API qtam_status qtam_frame_operator(qtam_plan_t plan, uint64_t plane_mask, 
  * and keeps the fastest with qtam_plan_set_variant. */
 QTAM_API qtam_status qtam_plan_variants(qtam_plan_t plan, int32_t* ids, int32_t capacity, int32_t* count);
 
-/* Select the row-kernel variant for subsequent calls on this plan.  Not
- * synchronised with calls running concurrently on other threads. */
+/* Select the row-kernel variant for subsequent calls on this plan (-1: the
+ * kernels of its own length again).  Not synchronised with calls running
+ * concurrently on other threads.  Streams (qtam_stream_*) of FP32 bisquare
+ * plans, the single-tile inverse and the tensor-core short DFT have kernels of
+ * their own, whichever variant is selected. */
 QTAM_API qtam_status qtam_plan_set_variant(qtam_plan_t plan, int32_t variant);
+
+/* The row-kernel variant the plan's launches run: the one selected last, -1
+ * (the kernels of the plan's own length) on a new plan.  Reading it and
+ * selecting it again later restores the plan. */
+QTAM_API qtam_status qtam_plan_running_variant(qtam_plan_t plan, int32_t* variant);
 
 /* Describe a variant: a name (radices, rows per block, occupancy target)
  * into name[capacity], threads per block and rows per block. */

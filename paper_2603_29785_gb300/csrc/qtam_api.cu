@@ -1027,6 +1027,12 @@ qtam_status qtam_plan_set_variant(qtam_plan_t pl, int32_t id) {
   return QTAM_OK;
 }
 
+qtam_status qtam_plan_running_variant(qtam_plan_t pl, int32_t* id) {
+  if (!pl || !id) return fail(QTAM_ERR_INVALID_ARG, "NULL argument");
+  *id = pl->rc.chosen ? pl->rc.variant : -1;
+  return QTAM_OK;
+}
+
 qtam_status qtam_variant_describe(int32_t id, char* name, size_t capacity, int32_t* threads, int32_t* rows_per_block) {
   if (id == -1) {
     if (name && capacity) std::snprintf(name, capacity, "the length's own kernels");

@@ -92,6 +92,7 @@ SIGNATURES = {
     "qtam_workspace_size": (ctypes.c_int, [_P, _I64, ctypes.POINTER(_SZ)]),
     "qtam_plan_variants": (ctypes.c_int, [_P, _P, ctypes.c_int32, ctypes.POINTER(ctypes.c_int32)]),
     "qtam_plan_set_variant": (ctypes.c_int, [_P, ctypes.c_int32]),
+    "qtam_plan_running_variant": (ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int32)]),
     "qtam_variant_describe": (ctypes.c_int, [ctypes.c_int32, ctypes.c_char_p, _SZ, ctypes.POINTER(ctypes.c_int32),
                                              ctypes.POINTER(ctypes.c_int32)]),
     "qtam_forward": (ctypes.c_int, [_P, _P, _I64, _P, _P, _SZ, _P]),
@@ -260,6 +261,12 @@ def qtam_plan_variants(plan) -> list[int]:
 
 def qtam_plan_set_variant(plan, variant: int):
     _check(lib().qtam_plan_set_variant(plan, int(variant)))
+
+
+def qtam_plan_running_variant(plan) -> int:
+    v = ctypes.c_int32()
+    _check(lib().qtam_plan_running_variant(plan, ctypes.byref(v)))
+    return v.value
 
 
 def qtam_variant_describe(variant: int) -> dict:
