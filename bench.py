@@ -707,7 +707,7 @@ def run_bank(args, local):
     out = {}
     for label, kw in (("bank", dict(window=wins, window_param=prms)), ("bisquare", {})):
         p = qtam.Plan(W["fs"], W["N"], W["qs"], W["fmin"], W["fmax"], W["K"], device=local, **kw)
-        qtune.tune(p, B)
+        tuned = qtune.tune(p, B)
         y = p.forward(x)
         xh = p.inverse(y)
         energy = torch.empty((B, p.P), dtype=torch.float64, device=x.device)
@@ -731,7 +731,7 @@ def run_bank(args, local):
         ms_m = ev[1].elapsed_time(ev[2]) / args.steps
         env_bytes = B * p.info["envelope_bytes_per_segment"]
         out[label] = {"msamples_per_s": round(B * W["N"] / ms / 1e3, 1), "ms_per_step": round(ms, 4),
-                      "row_variant": qtam.qtam_variant_describe(p.info["row_variant"])["name"],
+                      "row_variant": tuned["name"],
                       "plane_metrics_ms": round(ms_m, 4),
                       "plane_metrics_GB_s": round(env_bytes / (ms_m * 1e-3) / 1e9, 1),
                       "best_plane_by_energy_seg0": int(torch.argmax(energy[0]).item())}
