@@ -200,16 +200,37 @@ def run_reference(args, rank):
     print(json.dumps(line), flush=True)
 
 
-def measured_traffic(kernel: str):
-    """DRAM bytes per full-size launch from the committed ncu capture, or None
-    when the kernel sources changed since the counters were taken."""
+CSRC = os.path.join(ROOT, "paper_2603_29785_gb300", "csrc")
+
+
+def row_kernel_sources(csrc: str = CSRC):
+    """The files the row kernels are compiled from: the kernels of each length,
+    what launches them, and every file of the folder those include."""
+    import re
+    seen, todo = set(), ["kernels_any.cu", "kernels_rows.cu"]
+    while todo:
+        f = todo.pop()
+        if f not in seen and not os.path.dirname(f) and os.path.exists(os.path.join(csrc, f)):
+            seen.add(f)
+            todo += re.findall(r'^\s*#include "([^"]+)"', open(os.path.join(csrc, f)).read(), re.M)
+    return sorted(seen)
+
+
+def row_kernel_digest(csrc: str = CSRC) -> str:
     import hashlib
+    h = hashlib.sha256()
+    for f in row_kernel_sources(csrc):
+        h.update(open(os.path.join(csrc, f), "rb").read())
+    return h.hexdigest()
+
+
+def measured_traffic(kernel: str, variant: int):
+    """DRAM bytes per full-size launch from the committed ncu capture, or None
+    when the kernel sources changed since the counters were taken or the plan
+    runs another variant than they were taken of."""
     try:
         tr = json.load(open(os.path.join(ROOT, "profiles", "traffic.json")))
-        h = hashlib.sha256()
-        for f in ("kernels_rows.cu", "rows_common.cuh", "fft_static.cuh", "fft_core.cuh", "qtam_internal.h"):
-            h.update(open(os.path.join(ROOT, "paper_2603_29785_gb300", "csrc", f), "rb").read())
-        if h.hexdigest() != tr.get("source_sha256"):
+        if row_kernel_digest() != tr.get("source_sha256") or variant != tr.get("variant"):
             return None
         return tr.get(kernel, {}).get("bytes_per_launch_full")
     except (OSError, ValueError):
@@ -405,7 +426,7 @@ def run_gpu(args, rank, world, local):
         kernels[nm] = {"ms": round(float(t), 4), "alg_bytes": int(b), "GB_s": round(b / (t * 1e-3) / 1e9, 1)}
     dom = int(np.argmax(stage_avg_ms[1:3])) + 1
     achieved = stage_bytes[dom] / (stage_avg_ms[dom] * 1e-3) / 1e9
-    traffic = measured_traffic(["", "k_rows_forward", "k_rows_inverse"][dom])
+    traffic = measured_traffic(["", "k_rows_forward", "k_rows_inverse"][dom], qtam.qtam_plan_running_variant(p.handle))
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": hbm_peak, "unit": "GB/s",
                 "frac": round(achieved / hbm_peak, 4), "traffic": traffic, "kernel": stage_names[dom],
                 "peak_source": peak_src}
