@@ -659,7 +659,7 @@ def run_dense(args, local):
     fs, N, qs, K, eps = 4096.0, 8192, (4.0, 8.0, 16.0), 64, 1e-3
     B = args.batch * 4
     p = qtam.Plan(fs, N, qs, 20.0, 2048.0, K, stopband_eps=eps, remodulate=True, device=local)
-    tuned = qtune.tune(p, B)      # the compile-time variants built for the dense mode (M = 4320)
+    tuned = qtune.tune(p, B)      # the length's own kernels and the variants built for the dense mode (M = 4320)
     xh_ = np.stack([synth.glitchy_segment(500 + b, N, fs, chirp=(b % 2 == 0)) for b in range(B)]).astype(np.float32)
     x = torch.from_numpy(xh_).cuda()
     y = p.forward(x)
@@ -798,8 +798,8 @@ def run_serving(args, local):
 
 def precision_leg(args, local, B):
     """Precision sweep on the 64 s workload: envelope storage FP32 / BF16 / FP16
-    at M = 4800 (CUDA-core FFTs), and at M = 8192 the CUDA-core runtime engine
-    against the tensor-core short DFT (64 x 128 four-step on tcgen05, BF16
+    at M = 4800 (CUDA-core FFTs), and at M = 8192 the CUDA-core kernels against
+    the tensor-core short DFT (64 x 128 four-step on tcgen05, BF16
     operands, both directions): error against the FP64 oracle (2 segments),
     fwd+inv throughput, and the envelope and accumulation stages alone (64
     segments)."""

@@ -192,11 +192,11 @@ QTAM_API qtam_status qtam_plan_rows(qtam_plan_t plan, double* f, int64_t* kc, in
 QTAM_API qtam_status qtam_frame_operator(qtam_plan_t plan, uint64_t plane_mask, double* p_out);
 
 /* Row-kernel variants (launch shapes) usable for this plan: the kernels of the
- * plan's own length (-1, the ones a new plan runs; the runtime mixed-radix
- * engine for FP64 compute) and the variants registered for that length (FP32
- * compute).  Writes up to `capacity` ids
- * into `ids` and the total into *count.  All variants compute the same
- * transform; they differ in radix sequence, rows per block and occupancy.
+ * plan's own length (-1, the ones a new plan runs; with FP64 compute those of
+ * bisquare bands, and the runtime mixed-radix engine for other windows and
+ * the dense mode) and the variants registered for that length (FP32
+ * compute).  Writes up to `capacity` ids into `ids` and the total into *count.
+ * All variants compute the same transform; they differ in radix sequence, rows per block and occupancy.
  * An autotuner times them (qtam_stage_envelopes / qtam_stage_accumulate)
  * and keeps the fastest with qtam_plan_set_variant. */
 QTAM_API qtam_status qtam_plan_variants(qtam_plan_t plan, int32_t* ids, int32_t capacity, int32_t* count);
@@ -277,7 +277,8 @@ QTAM_API qtam_status qtam_roundtrip_host(qtam_plan_t plan, const void* x_host, i
 /* Signal-quality metrics per Q-plane for optimal-plane selection (App. A,
  * multi-Q bank, "optimal selection" mode): for every segment b and plane p,
  * energy[b*P + p] = sum over rows and columns of |Y|^2 (accumulated in FP64)
- * and peak[b*P + p] = max |Y|^2.  The plane with the largest energy (or peak)
+ * and peak[b*P + p] = max |Y|^2.  A NaN in the plane makes its energy NaN;
+ * the peak is that of the other values (0 without any).  The plane with the largest energy (or peak)
  * of each segment is its optimal plane.  energy (double) and peak (float) are
  * device arrays of batch*P entries. */
 QTAM_API qtam_status qtam_plane_metrics(qtam_plan_t plan, const void* y, int64_t batch, double* energy, float* peak,
@@ -285,7 +286,8 @@ QTAM_API qtam_status qtam_plane_metrics(qtam_plan_t plan, const void* y, int64_t
 
 /* The optimal plane of every segment from those metrics: best_energy[b] and
  * best_peak[b] (int64) are the first plane with the largest energy and peak of
- * segment b; a NaN counts as larger than any number. */
+ * segment b; a NaN counts as larger than any number (a peak of
+ * qtam_plane_metrics never is one). */
 QTAM_API qtam_status qtam_best_planes(qtam_plan_t plan, const double* energy, const float* peak, int64_t batch,
                              int64_t* best_energy, int64_t* best_peak, void* stream);
 

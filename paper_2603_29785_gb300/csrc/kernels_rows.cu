@@ -24,16 +24,15 @@
 // 141; 1200 (48 x 384) 55 + 58 against 57 + 65; 600 (96 x 384) 47 + 55 against 51
 // + 60; 300 (128 x 384) 35 + 41 against 35 + 47; 150 (200 x 384) 29 + 35 against
 // 33 + 45; 75 (400 x 384) 45 + 37 against 49 + 62; 8192 (16 x 640) 248 + 201
-// against 252 + 230.  FP64 plans run the runtime mixed-radix engine.
+// against 252 + 230.  FP64 plans run kernels_f64.cu for bisquare bands and the runtime
+// mixed-radix engine for window tables and dense tiles.
 #include "rows_common.cuh"
 
 namespace qtam {
 namespace {
 
-// StaticEngine<M, log2 rows per block, min blocks per SM, radices...>; the
-// first variant listed for a length is the default before tuning.
-// QTAM_VT: also built for window tables (the first such variant of a length
-// is the default of non-bisquare plans).
+// StaticEngine<M, log2 rows per block, min blocks per SM, radices...>.
+// QTAM_VT: also built for window tables.
 #define QTAM_V(M, NBS, MINB, ...) \
   make_variant<StaticEngine<M, NBS, MINB, __VA_ARGS__>>(#M ":" #__VA_ARGS__ " rows/blk 2^" #NBS " minblk " #MINB)
 #define QTAM_VT(M, NBS, MINB, ...) \
@@ -110,8 +109,9 @@ __global__ void __launch_bounds__(256) k_zero(uint2* p, int64_t words) {
 // block per part spent 48 FP64 instructions on two or three elements a thread (128 x 5
 // planes of 62 x 675: 186 us, 14 % of HBM).  A block takes `parts` consecutive parts, as
 // many as leave several waves, and reduces once, in one warp from shared memory (13 FP64
-// instructions, not 48); a partial widens to FP64 in the integer pipe.  scan of those
-// planes 145 -> 137 us, 378 before parts were joined.
+// instructions, not 48); a partial widens to FP64 in the integer pipe.  Joining the parts
+// took the kernel from 186 to 61 us, the one-warp reduction a scan of those planes from
+// 145 to 137 us.  A NaN makes the energy NaN and is left out of the peak (fmaxf).
 constexpr int kMetricParts = 64;
 
 // (double)x of a sum of squares; normal numbers by moving exponent and fraction

@@ -23,7 +23,7 @@ namespace {
 // 64-thread block; 0.087 at 4 rows per block), M = 300 0.054 against 0.066
 // ms (2 rows per block, 12 blocks per SM), M = 150 0.049 against 0.053 ms;
 // at M = 75 the two shapes trade places with the sample rate, so the older
-// one stays the default.  Fewer rows per block with more blocks per SM won
+// one stays listed first.  Fewer rows per block with more blocks per SM won
 // at every short length: a block's barrier then waits on fewer threads.  At
 // M = 8192 (64 s segments, Q {4..64} x 128 rows, 64 segments, FP32
 // envelopes) 16·8·8·8 at 2 blocks per SM takes 1.010 + 0.889 ms against
@@ -33,8 +33,9 @@ namespace {
 // 0.132 + 0.144 against 0.144 + 0.168 ms for 55 segments at 16384 Hz.  The
 // 4800-point kernel on 160 threads (two rounds in every stage, 114-117
 // registers) lost: 0.560 + 0.857 against 0.509 + 0.487 ms.  The first
-// preferred entry of a length is its default for bisquare plans; the tuner
-// times all of them.
+// preferred entry of a length is the one a plan's info names; the tuner times all
+// of them and the kernels of the length itself, which were faster than each
+// (kernels_rows.cu).
 template <class Eng> RowVariant make_variant_pref(const char* name) {
   RowVariant v = make_variant<Eng>(name);
   v.preferred = 1;

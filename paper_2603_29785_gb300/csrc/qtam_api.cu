@@ -371,8 +371,6 @@ bool choose_long(int64_t n, bool dbl, LongCfg& lc) {
       lc.row_nbs = rn;
       lc.rp1 = r1;
       lc.rp2 = r2;
-      lc.col_threads = t1;
-      lc.row_threads = t2;
       lc.col_smem = s1;
       lc.row_smem = s2;
     }
@@ -913,8 +911,8 @@ qtam_status qtam_plan(const qtam_plan_desc* d, int device, qtam_plan_t* out) {
   pl->rc.floor = pl->eps > 0;
   pl->rc.dense = (pl->eps > 0 && pl->remod) ? 2 : (pl->eps > 0 || pl->remod) ? 1 : 0;
   if (!dbl) {
-    // the first usable variant marked preferred for this length, else the
-    // first registered usable one
+    // what qtam_plan_info names before one is chosen: the first usable variant marked
+    // preferred for this length, else the first registered usable one
     for (int pass = 0; pass < 2 && pl->rc.variant < 0; ++pass)
       for (int v = 0; v < row_variant_count(); ++v)
         if (variant_usable(pl, v) && (pass == 1 || row_variant(v)->preferred)) {

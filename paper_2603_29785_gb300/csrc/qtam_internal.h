@@ -109,7 +109,6 @@ struct LongCfg {
   int col_nbs;  // log2 of columns per column-pass block
   int row_nbs;  // log2 of rows per row-pass block
   RadixPlan rp1, rp2;
-  int col_threads, row_threads;
   size_t col_smem, row_smem;
 };
 
@@ -254,7 +253,7 @@ struct RowVariant {
   RowFwdDenseFn fwd_dense;   // null unless built for the dense mode
   RowInvDenseFn inv_dense;
   int tw_pair = 0;   // stage tables in the row-pair format (c, c, s, s) per entry (kernels_rows_pair.cu)
-  int preferred = 0;   // default of its length for bisquare plans ahead of the other variants
+  int preferred = 0;   // named by the info of its length's bisquare plans ahead of the other variants
 };
 // the dense-mode variants live in their own translation unit (kernels_rows_dense.cu)
 int dense_row_variant_count();

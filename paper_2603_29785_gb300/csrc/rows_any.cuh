@@ -1,6 +1,7 @@
-// Row kernels with the whole launch shape fixed at compile time and the plan's
-// options chosen at run time: one forward and one inverse kernel per envelope
-// length serve every storage type, window family and dense-mode option.
+// Row kernels with the whole launch shape fixed at compile time.  Each envelope
+// length has a pair of kernels (forward, inverse) per AnyMode, which takes every
+// storage type and the carrier at run time, one pair for FP32 envelopes and bisquare
+// bands, and one pair for overlap-save columns.
 //
 // A block transforms NB rows that lie side by side in shared memory (row b at
 // b * PITCH): item w of a stage is butterfly j = w mod (M / R) of row

@@ -1,9 +1,9 @@
 """Autotuner for the row kernels' launch shapes.
 
 Every plan can run its per-row transforms with the kernels built for its
-envelope length M (variant -1; FP64: the runtime mixed-radix engine) or with any
-variant registered for that length (radix sequence, rows per block, occupancy
-target; see ``qtam_plan_variants``).  All
+envelope length M (variant -1; the only choice in FP64) or with any variant
+registered for that length (radix sequence, rows per block, occupancy target; see
+``qtam_plan_variants``).  Streams of FP32 bisquare plans always run the former.  All
 variants compute the same numbers; ``tune`` times each one on the plan's own
 shapes (the envelope stage and the accumulation stage, CUDA events on the
 current stream, synthetic inputs), keeps the fastest with
