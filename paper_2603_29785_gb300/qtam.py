@@ -160,13 +160,19 @@ def _ptr(t) -> int | None:
     raise TypeError(f"cannot pass {type(t)} as a pointer")
 
 
+def _current_stream(device: int) -> int:
+    """Handle of a device's current stream, without a Stream object per call where PyTorch has the lookup."""
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)     # absent from host-only PyTorch
+    if raw is not None and torch.cuda.is_initialized():
+        return raw(device)
+    return torch.cuda.current_stream(device).cuda_stream
+
+
 def _stream(stream) -> int | None:
     if stream is None:
         import torch
-        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)     # absent from host-only PyTorch
-        if raw is not None and torch.cuda.is_initialized():
-            return raw(torch.cuda.current_device())    # without a Stream object per call
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream(torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -434,13 +440,11 @@ def _empty(shape, dtype, device, stream=None):
     kernels queued on it.  It is also recorded on the current stream, where the caller will read it, so that
     dropping it waits for both."""
     import torch
-    if stream is None:
+    st = None if stream is None else _stream(stream) or 0
+    if st is None or st == _current_stream(device):
         return torch.empty(shape, dtype=dtype, device=f"cuda:{device}")
     dev = torch.device("cuda", device)
-    st = _stream(stream) or 0
     cur = torch.cuda.current_stream(dev)
-    if cur.cuda_stream == st:
-        return torch.empty(shape, dtype=dtype, device=dev)
     with torch.cuda.stream(torch.cuda.ExternalStream(st, device=dev) if st else torch.cuda.default_stream(dev)):
         t = torch.empty(shape, dtype=dtype, device=dev)
     t.record_stream(cur)
