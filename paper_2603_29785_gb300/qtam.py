@@ -489,7 +489,7 @@ class Plan:
         r = qtam_plan_rows(self.handle, self.P * self.K)
         shp = (self.P, self.K)
         self.geometry = Geometry(r["f"].reshape(shp), r["kc"].reshape(shp), r["h"].reshape(shp), r["c"].reshape(shp))
-        self._ws = threading.local()   # .by_stream: this thread's scratch, {stream handle: tensor}
+        self._ws = {}            # scratch: {(thread, stream handle): tensor}
         self._need = (None, 0)   # workspace bytes of the last batch size asked for
 
     def __del__(self):
@@ -506,27 +506,20 @@ class Plan:
         """(scratch tensor, its bytes) for `batch` segments on `stream` (default: the current one).
 
         Calls that may run at the same time need scratch of their own, so a plan keeps one buffer for
-        each stream a thread uses (at most MAX_SCRATCH a thread, the oldest given back first): work on
-        one stream is ordered, and two threads may interleave the kernels of their calls on one.  A
-        buffer is allocated on its stream, so that dropping it is ordered with the kernels using it."""
+        each stream a thread uses: work on one stream is ordered, and two threads may interleave the
+        kernels of their calls on one.  It is kept as long as the plan, whose tables a captured call needs
+        as well, unless a larger batch on its stream replaces it: capture the largest first.  A buffer
+        is allocated on its stream, so that dropping it is ordered with the kernels using it."""
         last, need = self._need
         if last != batch:
             need = qtam_workspace_size(self.handle, batch)
             self._need = (batch, need)
         st = _stream(stream) or 0
-        try:
-            mine = self._ws.by_stream
-        except AttributeError:
-            mine = self._ws.by_stream = {}
-        ws = mine.get(st)
+        key = (threading.get_ident(), st)
+        ws = self._ws.get(key)
         if ws is None or ws.numel() < need:
-            mine.pop(st, None)
-            while len(mine) >= self.MAX_SCRATCH:
-                del mine[next(iter(mine))]
-            ws = mine[st] = self._scratch(max(need, 256), st)
+            ws = self._ws[key] = self._scratch(max(need, 256), st)
         return ws, ws.numel()
-
-    MAX_SCRATCH = 32     # as many streams as PyTorch's pool hands out
 
     def _scratch(self, nbytes, st):
         import torch

@@ -116,3 +116,30 @@ def test_outputs_belong_to_the_stream_that_writes_them():
     assert y.data_ptr() != at
     torch.cuda.synchronize()
     assert torch.equal(twice, want + want)
+
+
+def test_replay_after_the_capturing_thread_has_ended():
+    """The scratch a captured call recorded is not given to anyone else while the plan lives."""
+    p = qtam.Plan(*ARGS, device=0)
+    x, other = inputs(p, 2)
+    want = p.forward(x)
+    made = {}
+
+    def capture():
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            p.forward(other)                              # this thread's scratch on s, before the capture
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            made["y"] = p.forward(x)
+        made.update(g=g, s=s, ws=p.workspace(6, s)[0].data_ptr())
+
+    t = threading.Thread(target=capture)
+    t.start()
+    t.join()
+    with torch.cuda.stream(made["s"]):                    # new blocks of that stream's pool are others
+        taken = [torch.empty(p.workspace(6, 0)[1], dtype=torch.uint8, device="cuda") for _ in range(4)]
+    assert made["ws"] not in [b.data_ptr() for b in taken]
+    made["g"].replay()
+    assert torch.equal(made["y"], want)

@@ -34,16 +34,23 @@ def test_each_stream_and_thread_has_its_own(plan):
     assert plan.workspace(4, 11)[0] is a
 
 
-def test_growth_and_bound(plan):
+def test_growth(plan):
     a, _ = plan.workspace(1, 5)
     b, nb = plan.workspace(9, 5)
     assert b is not a and nb >= qtam.qtam_workspace_size(plan.handle, 9)
     assert plan.workspace(1, 5)[0] is b
-    first, _ = plan.workspace(1, 100)
-    for s in range(101, 100 + plan.MAX_SCRATCH):
+
+
+def test_scratch_lives_as_long_as_the_plan(plan):
+    """A graph captured by a thread that has ended, or before many other streams were used, still replays on it."""
+    import weakref
+    refs = [weakref.ref(plan.workspace(1, 5)[0])]
+    t = threading.Thread(target=lambda: refs.append(weakref.ref(plan.workspace(1, 6)[0])))
+    t.start()
+    t.join()
+    for s in range(100, 200):
         plan.workspace(1, s)
-    assert plan.workspace(1, 100)[0] is first and plan.workspace(1, 5)[0] is not b     # the oldest went first
-    assert len(plan._ws.by_stream) == plan.MAX_SCRATCH
+    assert all(r() is not None for r in refs)
 
 
 class FakeTensor:
